@@ -49,6 +49,12 @@ constexpr float E1 = -277.0f / 64512.0f, E3 = 6925.0f / 370944.0f, E4 = -6925.0f
 struct F3 { float x, y, z; };
 struct DF { float hi, lo; };
 
+// One rounding each, never contracted with a neighbour: the attempt's arithmetic is written out in
+// these, so that every instantiation and every arrangement of the code gives the same bits.
+__device__ __forceinline__ float fm(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
+
 // a + b with the rounding error carried in lo (Knuth TwoSum, then renormalise).
 __device__ __forceinline__ DF df_add(DF a, float b) {
     const float s = a.hi + b;
@@ -114,42 +120,49 @@ __device__ __forceinline__ F3 corner_f(const FieldF& F, int node) {
 template <int L>
 constexpr bool kBF16 = (L == LAYOUT_BF16X4 || L == LAYOUT_BF16_CELLS);
 
-// 256-bit read-only loads: the cell-major layouts hold a cell's 8 corners in 96 B (FP32) or
-// 64 B (BF16), 32-byte aligned, so a lookup takes 3 or 2 loads instead of 8 scattered ones.
-__device__ __forceinline__ void ld8(const void* p, unsigned (&w)[8]) {
-    asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]),
-                   "=r"(w[7])
-                 : "l"(p));
+// The corners of the cell a lane last looked up, as the cell-major copy holds them (96 B FP32 or
+// 64 B BF16, 32-byte aligned: 3 or 2 256-bit loads instead of 8 scattered ones). They stay in
+// registers, and a lookup in the same cell loads nothing: consecutive stages of an attempt lie
+// 0.1 to 0.4 steps apart, so about three of four find their cell there. The kernel is bound by the
+// latency of the six dependent lookups, and with fewer lanes per load L1 answers sooner (10^6
+// nuclei on 256^3 over 100 Mpc: 80.8 -> 75.1 ms; modulated 220^3 x 128^3: 79.5 -> 74.6 ms).
+template <int L>
+struct Cell {
+    static constexpr int kWords = (L == LAYOUT_F32_CELLS) ? 24 : 16;
+    unsigned w[kWords];
+    int id;   // cell index in the grid of the lane's particle, -1: none
+};
+
+// 256-bit read-only load into w where on is non-zero; w is left as it is elsewhere.
+__device__ __forceinline__ void ld8_if(int on, const void* p, unsigned* w) {
+    asm("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %8, 0;\n\t"
+        "@q ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%9];\n\t}"
+        : "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3]), "+r"(w[4]), "+r"(w[5]), "+r"(w[6]), "+r"(w[7])
+        : "r"(on), "l"(p));
 }
 
-// The 8 corners of a cell from a cell-major copy, in the order 000, 001, ..., 111 (the same
-// values corner_f reads from the node layout).
+// The 8 corners of a cell in the order 000, 001, ..., 111 (the same values corner_f reads from
+// the node layout).
 template <int L>
-__device__ __forceinline__ void cell_corners(const FieldF& F, long long cell, F3& g0, F3& g1, F3& g2, F3& g3,
+__device__ __forceinline__ void cell_corners(const FieldF& F, int cell, Cell<L>& cc, F3& g0, F3& g1, F3& g2, F3& g3,
                                              F3& g4, F3& g5, F3& g6, F3& g7) {
+    const int other = cell != cc.id;
+    cc.id = cell;
+    const char* q = static_cast<const char*>(F.data) + (long long)cell * (Cell<L>::kWords * 4);
+#pragma unroll
+    for (int k = 0; k < Cell<L>::kWords; k += 8) ld8_if(other, q + 4 * k, cc.w + k);
     if constexpr (L == LAYOUT_F32_CELLS) {
-        const unsigned* q = static_cast<const unsigned*>(F.data) + cell * 24;
-        unsigned a[8], b[8], c[8];
-        ld8(q, a);
-        ld8(q + 8, b);
-        ld8(q + 16, c);
-        auto f = [](unsigned u) { return __uint_as_float(u); };
-        g0 = {f(a[0]), f(a[1]), f(a[2])}; g1 = {f(a[3]), f(a[4]), f(a[5])};
-        g2 = {f(a[6]), f(a[7]), f(b[0])}; g3 = {f(b[1]), f(b[2]), f(b[3])};
-        g4 = {f(b[4]), f(b[5]), f(b[6])}; g5 = {f(b[7]), f(c[0]), f(c[1])};
-        g6 = {f(c[2]), f(c[3]), f(c[4])}; g7 = {f(c[5]), f(c[6]), f(c[7])};
+        auto c3 = [&](int c) {
+            return F3{__uint_as_float(cc.w[3 * c]), __uint_as_float(cc.w[3 * c + 1]), __uint_as_float(cc.w[3 * c + 2])};
+        };
+        g0 = c3(0); g1 = c3(1); g2 = c3(2); g3 = c3(3); g4 = c3(4); g5 = c3(5); g6 = c3(6); g7 = c3(7);
     } else {
         // BF16: per corner two words, (x | y << 16) and (z | pad << 16)
-        const unsigned* q = static_cast<const unsigned*>(F.data) + cell * 16;
-        unsigned a[8], b[8];
-        ld8(q, a);
-        ld8(q + 8, b);
-        auto c3 = [](unsigned w0, unsigned w1) {
+        auto c3 = [&](int c) {
+            const unsigned w0 = cc.w[2 * c], w1 = cc.w[2 * c + 1];
             return F3{__uint_as_float(w0 << 16), __uint_as_float(w0 & 0xFFFF0000u), __uint_as_float(w1 << 16)};
         };
-        g0 = c3(a[0], a[1]); g1 = c3(a[2], a[3]); g2 = c3(a[4], a[5]); g3 = c3(a[6], a[7]);
-        g4 = c3(b[0], b[1]); g5 = c3(b[2], b[3]); g6 = c3(b[4], b[5]); g7 = c3(b[6], b[7]);
+        g0 = c3(0); g1 = c3(1); g2 = c3(2); g3 = c3(3); g4 = c3(4); g5 = c3(5); g6 = c3(6); g7 = c3(7);
     }
 }
 
@@ -186,16 +199,16 @@ __device__ __forceinline__ double origin(const PropArgs& a, int gid, int c) {
 // Trilinear weights and the corner sum, in the same order for the cached and gathered paths.
 __device__ __forceinline__ float trilerp(float fx, float fy, float fz, float m0, float m1, float m2,
                                          float m3, float m4, float m5, float m6, float m7) {
-    const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
-    const float w00 = gx * gy, w01 = gx * fy, w10 = fx * gy, w11 = fx * fy;
-    float v = (w00 * gz) * m0;
-    v = fmaf(w00 * fz, m1, v);
-    v = fmaf(w01 * gz, m2, v);
-    v = fmaf(w01 * fz, m3, v);
-    v = fmaf(w10 * gz, m4, v);
-    v = fmaf(w10 * fz, m5, v);
-    v = fmaf(w11 * gz, m6, v);
-    v = fmaf(w11 * fz, m7, v);
+    const float gx = __fsub_rn(1.0f, fx), gy = __fsub_rn(1.0f, fy), gz = __fsub_rn(1.0f, fz);
+    const float w00 = mul(gx, gy), w01 = mul(gx, fy), w10 = mul(fx, gy), w11 = mul(fx, fy);
+    float v = mul(mul(w00, gz), m0);
+    v = fm(mul(w00, fz), m1, v);
+    v = fm(mul(w01, gz), m2, v);
+    v = fm(mul(w01, fz), m3, v);
+    v = fm(mul(w10, gz), m4, v);
+    v = fm(mul(w10, fz), m5, v);
+    v = fm(mul(w11, gz), m6, v);
+    v = fm(mul(w11, fz), m7, v);
     return v;
 }
 
@@ -232,8 +245,8 @@ __device__ __forceinline__ void mod_fill(float* sm, const FieldDev& G, int bx, i
 // lookup on the scalar grid, with the offset converted to modulation cells.
 __device__ __forceinline__ float modulation_f(const FieldDev* fields, int gid, float* sm, const MF& m, F3 p) {
     float fx, fy, fz;
-    const int cx = floor_frac(fmaf(p.x, m.q, m.f0.x), fx), cy = floor_frac(fmaf(p.y, m.q, m.f0.y), fy),
-              cz = floor_frac(fmaf(p.z, m.q, m.f0.z), fz);
+    const int cx = floor_frac(fm(p.x, m.q, m.f0.x), fx), cy = floor_frac(fm(p.y, m.q, m.f0.y), fy),
+              cz = floor_frac(fm(p.z, m.q, m.f0.z), fz);
     // cell relative to the cached block's low corner: 0 or 1 when inside it
     const int jx = cx + (m.lo & 1), jy = cy + ((m.lo >> 1) & 1), jz = cz + ((m.lo >> 2) & 1);
     float m0, m1, m2, m3, m4, m5, m6, m7;
@@ -262,17 +275,16 @@ __device__ __forceinline__ float modulation_f(const FieldDev* fields, int gid, f
     return trilerp(fx, fy, fz, m0, m1, m2, m3, m4, m5, m6, m7);
 }
 
-// Trilinear periodic lookup at (base cell b, fraction f0) + offset p (cells); with M, times
-// the modulation value there. P2: the vector grid's sizes are powers of two, and the cell index
+// Trilinear periodic lookup at the local coordinate g (cells from the base cell b); with M, times
+// the modulation value at the offset p from the step start. P2: the vector grid's sizes are powers of two, and the cell index
 // wraps with a mask (the general wrap's integer modulo, inlined at each of an attempt's six
 // lookups and never run for such grids, stays out of the kernel: +8.6 % measured).
 template <int L, bool M, bool P2>
-__device__ __forceinline__ F3 field_f(const FieldF& F, int bx, int by, int bz, F3 f0,
+__device__ __forceinline__ F3 field_f(const FieldF& F, int bx, int by, int bz,
                                       const FieldDev* fields, int gid, float* sm, const MF& mf,
-                                      F3 p) {
+                                      Cell<L>& cc, F3 g, F3 p) {
     float fx, fy, fz;
-    const int cx = floor_frac(f0.x + p.x, fx), cy = floor_frac(f0.y + p.y, fy),
-              cz = floor_frac(f0.z + p.z, fz);
+    const int cx = floor_frac(g.x, fx), cy = floor_frac(g.y, fy), cz = floor_frac(g.z, fz);
     const int ix = P2 ? (bx + cx) & (F.nx - 1) : wrap(bx + cx, F.nx, F.pow2),
               iy = P2 ? (by + cy) & (F.ny - 1) : wrap(by + cy, F.ny, F.pow2),
               iz = P2 ? (bz + cz) & (F.nz - 1) : wrap(bz + cz, F.nz, F.pow2);
@@ -287,43 +299,28 @@ __device__ __forceinline__ F3 field_f(const FieldF& F, int bx, int by, int bz, F
         g4 = corner_f<L>(F, r10 + iz); g5 = corner_f<L>(F, r10 + iz1);
         g6 = corner_f<L>(F, r11 + iz); g7 = corner_f<L>(F, r11 + iz1);
     } else {
-        cell_corners<L>(F, ((long long)ix * F.ny + iy) * F.nz + iz, g0, g1, g2, g3, g4, g5, g6, g7);
+        cell_corners<L>(F, (ix * F.ny + iy) * F.nz + iz, cc, g0, g1, g2, g3, g4, g5, g6, g7);
     }
-    const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
-    const float w00 = gx * gy, w01 = gx * fy, w10 = fx * gy, w11 = fx * fy;
+    const float gx = __fsub_rn(1.0f, fx), gy = __fsub_rn(1.0f, fy), gz = __fsub_rn(1.0f, fz);
+    const float w00 = mul(gx, gy), w01 = mul(gx, fy), w10 = mul(fx, gy), w11 = mul(fx, fy);
     float w;
     F3 B;
-    w = w00 * gz; B.x = w * g0.x;          B.y = w * g0.y;          B.z = w * g0.z;
-    w = w00 * fz; B.x = fmaf(w, g1.x, B.x); B.y = fmaf(w, g1.y, B.y); B.z = fmaf(w, g1.z, B.z);
-    w = w01 * gz; B.x = fmaf(w, g2.x, B.x); B.y = fmaf(w, g2.y, B.y); B.z = fmaf(w, g2.z, B.z);
-    w = w01 * fz; B.x = fmaf(w, g3.x, B.x); B.y = fmaf(w, g3.y, B.y); B.z = fmaf(w, g3.z, B.z);
-    w = w10 * gz; B.x = fmaf(w, g4.x, B.x); B.y = fmaf(w, g4.y, B.y); B.z = fmaf(w, g4.z, B.z);
-    w = w10 * fz; B.x = fmaf(w, g5.x, B.x); B.y = fmaf(w, g5.y, B.y); B.z = fmaf(w, g5.z, B.z);
-    w = w11 * gz; B.x = fmaf(w, g6.x, B.x); B.y = fmaf(w, g6.y, B.y); B.z = fmaf(w, g6.z, B.z);
-    w = w11 * fz; B.x = fmaf(w, g7.x, B.x); B.y = fmaf(w, g7.y, B.y); B.z = fmaf(w, g7.z, B.z);
+    w = mul(w00, gz); B.x = mul(w, g0.x);     B.y = mul(w, g0.y);     B.z = mul(w, g0.z);
+    w = mul(w00, fz); B.x = fm(w, g1.x, B.x); B.y = fm(w, g1.y, B.y); B.z = fm(w, g1.z, B.z);
+    w = mul(w01, gz); B.x = fm(w, g2.x, B.x); B.y = fm(w, g2.y, B.y); B.z = fm(w, g2.z, B.z);
+    w = mul(w01, fz); B.x = fm(w, g3.x, B.x); B.y = fm(w, g3.y, B.y); B.z = fm(w, g3.z, B.z);
+    w = mul(w10, gz); B.x = fm(w, g4.x, B.x); B.y = fm(w, g4.y, B.y); B.z = fm(w, g4.z, B.z);
+    w = mul(w10, fz); B.x = fm(w, g5.x, B.x); B.y = fm(w, g5.y, B.y); B.z = fm(w, g5.z, B.z);
+    w = mul(w11, gz); B.x = fm(w, g6.x, B.x); B.y = fm(w, g6.y, B.y); B.z = fm(w, g6.z, B.z);
+    w = mul(w11, fz); B.x = fm(w, g7.x, B.x); B.y = fm(w, g7.y, B.y); B.z = fm(w, g7.z, B.z);
     if constexpr (M) {
         float m = modulation_f(fields, gid, sm, mf, p);
-        if constexpr (kBF16<L>) m *= F.scale;
-        B.x *= m; B.y *= m; B.z *= m;
+        if constexpr (kBF16<L>) m = mul(m, F.scale);
+        B.x = mul(B.x, m); B.y = mul(B.y, m); B.z = mul(B.z, m);
     } else if constexpr (kBF16<L>) {
-        B.x *= F.scale; B.y *= F.scale; B.z *= F.scale;
+        B.x = mul(B.x, F.scale); B.y = mul(B.y, F.scale); B.z = mul(B.z, F.scale);
     }
     return B;
-}
-
-struct Y { F3 p, u; };   // local position offset (cells) and direction
-
-template <int L, bool M, bool P2>
-__device__ __forceinline__ Y deriv_f(const FieldF& F, int bx, int by, int bz, F3 f0,
-                                     const FieldDev* fields, int gid, float* sm, const MF& mf,
-                                     float kappa, const Y& y) {
-    const F3 B = field_f<L, M, P2>(F, bx, by, bz, f0, fields, gid, sm, mf, y.p);
-    Y k;
-    k.p = y.u;
-    k.u.x = kappa * (y.u.y * B.z - y.u.z * B.y);
-    k.u.y = kappa * (y.u.z * B.x - y.u.x * B.z);
-    k.u.z = kappa * (y.u.x * B.y - y.u.y * B.x);
-    return k;
 }
 
 __device__ __forceinline__ float clampf_(float v, float lo, float hi) { return fminf(fmaxf(v, lo), hi); }
@@ -385,6 +382,10 @@ __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* s
     float h = 0, h_first = 0, h_propc = 0, h_int = 0, h_dist = 0, rl = 0, rpd = 0, kappa = 0;
     int rejected = 0;
     int att_step = 0;
+    Cell<L> cc;
+    cc.id = -1;
+#pragma unroll
+    for (int k = 0; k < Cell<L>::kWords; ++k) cc.w[k] = 0;
     unsigned acc_tot = 0, att_tot = 0, sec_tot = 0;
     unsigned bits = 0;
 
@@ -446,6 +447,7 @@ __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* s
             taken = 0;
             att_call = 0;
             new_step = true;
+            cc.id = -1;
         }
         if (__ballot_sync(kFull, slot >= 0) == 0) break;
 
@@ -519,35 +521,49 @@ __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* s
                 new_step = false;
             }
             // ---- one Cash-Karp attempt in the local frame (FP32) ----
-            const Y y0{{0.0f, 0.0f, 0.0f}, u};
-            const Y k1 = deriv_f<L, M, P2>(F, bx, by, bz, f0, a.fields, gid, sm, mf, kappa, y0);
-            Y t;
-#define STG(expr)                                                                              \
-            t.p.x = h * (expr(p.x)); t.p.y = h * (expr(p.y)); t.p.z = h * (expr(p.z));         \
-            t.u.x = fmaf(h, (expr(u.x)), u.x); t.u.y = fmaf(h, (expr(u.y)), u.y);               \
-            t.u.z = fmaf(h, (expr(u.z)), u.z);
-#define S2(c) (A21 * k1.c)
-            STG(S2)
-            const Y k2 = deriv_f<L, M, P2>(F, bx, by, bz, f0, a.fields, gid, sm, mf, kappa, t);
-#define S3(c) (A31 * k1.c + A32 * k2.c)
-            STG(S3)
-            const Y k3 = deriv_f<L, M, P2>(F, bx, by, bz, f0, a.fields, gid, sm, mf, kappa, t);
-#define S4(c) (A41 * k1.c + A42 * k2.c + A43 * k3.c)
-            STG(S4)
-            const Y k4 = deriv_f<L, M, P2>(F, bx, by, bz, f0, a.fields, gid, sm, mf, kappa, t);
-#define S5(c) (A51 * k1.c + A52 * k2.c + A53 * k3.c + A54 * k4.c)
-            STG(S5)
-            const Y k5 = deriv_f<L, M, P2>(F, bx, by, bz, f0, a.fields, gid, sm, mf, kappa, t);
-#define S6(c) (A61 * k1.c + A62 * k2.c + A63 * k3.c + A64 * k4.c + A65 * k5.c)
-            STG(S6)
-            const Y k6 = deriv_f<L, M, P2>(F, bx, by, bz, f0, a.fields, gid, sm, mf, kappa, t);
-#define SB(c) (B1 * k1.c + B3 * k3.c + B4 * k4.c + B6 * k6.c)
-#define SE(c) (E1 * k1.c + E3 * k3.c + E4 * k4.c + E5 * k5.c + E6 * k6.c)
-            const F3 dp{h * SB(p.x), h * SB(p.y), h * SB(p.z)};
-            const F3 du{h * SB(u.x), h * SB(u.y), h * SB(u.z)};       // direction increment
-            const F3 ex{SE(p.x), SE(p.y), SE(p.z)};                  // |dx| / h
-            const F3 eu{h * SE(u.x), h * SE(u.y), h * SE(u.z)};      // |du|
-#undef STG
+            F3 g = f0, p{0.0f, 0.0f, 0.0f}, tu = u;        // local coordinate, offset, direction
+            // kappa u x B at the stage
+            auto force = [&]() {
+                const F3 B = field_f<L, M, P2>(F, bx, by, bz, a.fields, gid, sm, mf, cc, g, p);
+                return F3{mul(kappa, fm(tu.y, B.z, -mul(tu.z, B.y))), mul(kappa, fm(tu.z, B.x, -mul(tu.x, B.z))),
+                          mul(kappa, fm(tu.x, B.y, -mul(tu.y, B.x)))};
+            };
+            // coordinate, offset and direction of the next stage from its sums
+            auto next = [&](F3 sp, F3 su) {
+                if constexpr (M) {
+                    p = {mul(h, sp.x), mul(h, sp.y), mul(h, sp.z)};
+                    g = {add(f0.x, p.x), add(f0.y, p.y), add(f0.z, p.z)};
+                } else {
+                    g = {fm(h, sp.x, f0.x), fm(h, sp.y, f0.y), fm(h, sp.z, f0.z)};
+                }
+                tu = {fm(h, su.x, u.x), fm(h, su.y, u.y), fm(h, su.z, u.z)};
+            };
+#define S2(q, c) mul(A21, q(1).c)
+#define S3(q, c) fm(A31, q(1).c, mul(A32, q(2).c))
+#define S4(q, c) fm(A43, q(3).c, fm(A41, q(1).c, mul(A42, q(2).c)))
+#define S5(q, c) fm(A54, q(4).c, fm(A53, q(3).c, fm(A52, q(2).c, mul(A51, q(1).c))))
+#define S6(q, c) fm(A65, q(5).c, fm(A64, q(4).c, fm(A63, q(3).c, fm(A61, q(1).c, mul(A62, q(2).c)))))
+#define SB(q, c) fm(B6, q(6).c, fm(B4, q(4).c, fm(B1, q(1).c, mul(B3, q(3).c))))
+#define SE(q, c) fm(E6, q(6).c, fm(E5, q(5).c, fm(E4, q(4).c, fm(E3, q(3).c, mul(E1, q(1).c)))))
+#define KP(n) k##n##p
+#define KU(n) k##n##u
+#define V3OF(S, q) F3{S(q, x), S(q, y), S(q, z)}
+            const F3 k1p = u, k1u = force();
+            next(V3OF(S2, KP), V3OF(S2, KU));
+            const F3 k2p = tu, k2u = force();
+            next(V3OF(S3, KP), V3OF(S3, KU));
+            const F3 k3p = tu, k3u = force();
+            next(V3OF(S4, KP), V3OF(S4, KU));
+            const F3 k4p = tu, k4u = force();
+            next(V3OF(S5, KP), V3OF(S5, KU));
+            const F3 k5p = tu, k5u = force();
+            next(V3OF(S6, KP), V3OF(S6, KU));
+            const F3 k6p = tu, k6u = force();
+            const F3 bp = V3OF(SB, KP), bu = V3OF(SB, KU), eu1 = V3OF(SE, KU);
+            const F3 dp{mul(h, bp.x), mul(h, bp.y), mul(h, bp.z)};
+            const F3 du{mul(h, bu.x), mul(h, bu.y), mul(h, bu.z)};      // direction increment
+            const F3 ex = V3OF(SE, KP);                                 // |dx| / h
+            const F3 eu{mul(h, eu1.x), mul(h, eu1.y), mul(h, eu1.z)};   // |du|
 #undef S2
 #undef S3
 #undef S4
@@ -555,10 +571,13 @@ __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* s
 #undef S6
 #undef SB
 #undef SE
+#undef KP
+#undef KU
+#undef V3OF
             att_step += 1;
             // ---- FP64 error norm and accept/reject (certified from FP32 outside the band) ----
-            const float qx32 = ex.x * ex.x + ex.y * ex.y + ex.z * ex.z;
-            const float qu32 = eu.x * eu.x + eu.y * eu.y + eu.z * eu.z;
+            const float qx32 = fm(ex.z, ex.z, fm(ex.x, ex.x, mul(ex.y, ex.y)));
+            const float qu32 = fm(eu.z, eu.z, fm(eu.x, eu.x, mul(eu.y, eu.y)));
             bool accept;
             if (qx32 <= tol2_lo && qu32 <= tol2_lo) {
                 accept = true;
@@ -572,7 +591,7 @@ __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* s
                 accept = fmax(qx, qu) <= tol2;
             }
             accept = accept || (h <= hmin_c);
-            const float r2 = fmaxf(qx32, qu32) * inv_tol2;
+            const float r2 = mul(fmaxf(qx32, qu32), inv_tol2);
             if (!accept) {
                 const float shrink = clampf_(0.95f * powf_pos(r2, -0.125f), 0.1f, 1.0f);
                 h = fmaxf(h * shrink, hmin_c);
@@ -670,7 +689,7 @@ __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* s
                     n_int = (int)kk;
                     tau = (float)(-crp_log(uniform01(a.seed, uid, kk, 0u)));
                 } else {
-                    tau = tau - h * rpd;
+                    tau = fm(-h, rpd, tau);
                 }
             }
             new_step = true;
