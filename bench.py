@@ -434,8 +434,8 @@ def roofline_for(form, attempted, accepted, tables, prop_s, calls=1, workload=""
     """Roofline of the propagate kernel for one form, from the live CUDA-event time."""
     terms = roofline_terms(form, attempted, accepted, tables, prop_s, modulated, grid_dtype,
                            grid_bytes, peaks)
-    kern = ("k_propagate_fp64" if form == "fp64" else "k_propagate_mixed") + \
-        " (2 launches per call + 4 bookkeeping kernels)"
+    kern = ("k_propagate_fp64, then k_propagate_fp64_team for what is left" if form == "fp64" else
+            "k_propagate_mixed, two launches") + " (and the bookkeeping kernels of a call)"
     return roofline_from_terms(terms, traffic_for(workload, form, attempted, calls), kern, note)
 
 

@@ -220,7 +220,7 @@ typedef struct {
     int32_t cadence;         /* attempts between refill checks; 0: default (2 in the precision form, 1 in FP64) */
     int64_t max_steps;       /* accepted steps per particle per call; <= 0: no limit */
     int32_t order;           /* work-list order: CRP_ORDER_* (0: default = CRP_ORDER_COST) */
-    int32_t pickup;          /* secondaries created in a launch: CRP_PICKUP_* (0: default = OFF) */
+    int32_t pickup;          /* secondaries created in a launch: CRP_PICKUP_* */
     int32_t grid_layout;     /* precision form: CRP_GRID_* (0: default = AUTO) */
     int32_t pad_;
 } crp_params;
@@ -230,7 +230,8 @@ typedef struct {
 #define CRP_ORDER_COST 2         /* lowest rigidity E/Z first: expected longest first */
 #define CRP_ORDER_GRID 3         /* by grid_id, then lowest rigidity first: concurrent particles
                                     share field realisations (cache locality over many grids) */
-#define CRP_PICKUP_DEFAULT 0
+#define CRP_PICKUP_DEFAULT 0     /* taken up as they come, before the rest of the work list: a secondary
+                                    inherits a low energy and can be the longest trajectory of the call */
 #define CRP_PICKUP_OFF 1         /* secondaries wait for the second launch */
 #define CRP_PICKUP_ON 2          /* idle warps take secondaries pushed earlier in the launch */
 int crp_propagate(crp_sim* sim, const crp_params* params, double tolerance, double min_step_m,

@@ -211,6 +211,10 @@ __global__ void k_prepare(Counters* C) {
     C->head[0] = 0;
     C->head[1] = 0;
     C->reserve = C->n_used;
+    C->cur = 0;
+    C->pushed = 0;
+    C->head0 = 0;
+    C->left = 0;
 }
 
 // ---- work list in order of expected cost (longest first) ------------------------------
@@ -326,15 +330,22 @@ __global__ void k_build_worklist(const int32_t* __restrict__ status, int32_t* __
     }
 }
 
-// After a propagate launch over list `from`: fix the slot count, reset the pop head and
-// the list that the next launch pushes into.
-__global__ void k_swap(Counters* C, long long capacity, int from) {
+// After a propagate launch over list C->cur: fix the slot count, reset the pop head and the list
+// that the next launch pushes into, and make the other list the next one. A one-lane launch that
+// left its list alone (at most min_work entries) changes nothing.
+__global__ void k_swap(Counters* C, long long capacity, long long min_work) {
     CRP_COUNT_RUN();
+    const int from = C->cur;
+    if ((long long)(C->count[from] - C->head0) <= min_work) return;
     const unsigned long long r = C->reserve;
     C->n_used = r < (unsigned long long)capacity ? r : (unsigned long long)capacity;
     C->reserve = C->n_used;
     C->head[from] = 0;      // the other list keeps its head: the next launch continues it
     C->count[from] = 0;
+    C->cur = 1 - from;
+    C->pushed = 1;
+    C->head0 = C->head[1 - from];
+    C->left = 0;
     C->launches += 1;
 }
 
@@ -413,6 +424,9 @@ struct Plan {
     PropArgs a{};
     int grid = 0, block = 0, order = 0, mixed = 0, n_buckets = 0, layout = 0, mod = 0;
     int p2 = 0;   // every field's vector grid has power-of-two sizes
+    int team_grid = 0, team_block = 0;   // three-lane kernel: blocks (0: not launched), threads per block
+    int team_launches = 0;
+    int lane_launches = 2;               // launches of the one-lane kernel before those
 };
 
 }  // namespace
@@ -449,6 +463,7 @@ struct crp_sim {
     int32_t* lists[2] = {nullptr, nullptr};
     int32_t* done_list = nullptr;
     Counters* ctr = nullptr;
+    int32_t* taken = nullptr;           // accepted steps of this call, for particles handed between launches
     unsigned* sort_scratch = nullptr;   // [hist n_buckets][offsets n_buckets]
     cudaStream_t last = nullptr;
     cudaGraph_t loop_graph = nullptr;   // crp_propagate_loop, cached for one plan
@@ -728,6 +743,9 @@ int crp_sim_create(const crp_field* const* fields, int32_t n_fields, const crp_t
     if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->lists[0], sizeof(int32_t) * capacity);
     if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->lists[1], sizeof(int32_t) * capacity);
     if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->done_list, sizeof(int32_t) * capacity);
+    if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->taken, sizeof(int32_t) * capacity);
+    for (int k = 0; k < 2; ++k)   // no entry published
+        if (rc == CRP_OK && e == cudaSuccess) e = cudaMemset(s->lists[k], 0xff, sizeof(int32_t) * capacity);
     if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->ctr, sizeof(Counters));
     if (rc == CRP_OK && e == cudaSuccess) e = cudaMemset(s->ctr, 0, sizeof(Counters));
     const size_t sort_bytes = 2 * (size_t)kBuckets * n_fields * sizeof(unsigned);
@@ -776,6 +794,7 @@ int crp_sim_destroy(crp_sim* s) {
     if (s->lists[0]) cudaFree(s->lists[0]);
     if (s->lists[1]) cudaFree(s->lists[1]);
     if (s->done_list) cudaFree(s->done_list);
+    if (s->taken) cudaFree(s->taken);
     if (s->ctr) cudaFree(s->ctr);
     if (s->sort_scratch) cudaFree(s->sort_scratch);
     if (s->loop_exec) cudaGraphExecDestroy(s->loop_exec);
@@ -805,10 +824,13 @@ int crp_sim_reserve(crp_sim* s, int64_t capacity) {
     SimState ns{};
     rc = alloc_state(ns, capacity);
     if (rc) return rc;
-    int32_t *l0 = nullptr, *l1 = nullptr, *dl = nullptr;
+    int32_t *l0 = nullptr, *l1 = nullptr, *dl = nullptr, *tk = nullptr;
     cudaError_t e = dev_malloc(&l0, sizeof(int32_t) * capacity);
+    if (e == cudaSuccess) e = dev_malloc(&tk, sizeof(int32_t) * capacity);
     if (e == cudaSuccess) e = dev_malloc(&l1, sizeof(int32_t) * capacity);
     if (e == cudaSuccess) e = dev_malloc(&dl, sizeof(int32_t) * capacity);
+    if (e == cudaSuccess) e = cudaMemset(l0, 0xff, sizeof(int32_t) * capacity);
+    if (e == cudaSuccess) e = cudaMemset(l1, 0xff, sizeof(int32_t) * capacity);
     for (int c = 0; c < CRP_N_COLS && e == cudaSuccess; ++c)
         e = cudaMemcpy(*col_ptr(ns, c), *col_ptr(s->st, c), (size_t)h.n_used * kCols[c].size,
                        cudaMemcpyDeviceToDevice);
@@ -819,12 +841,15 @@ int crp_sim_reserve(crp_sim* s, int64_t capacity) {
         if (l0) cudaFree(l0);
         if (l1) cudaFree(l1);
         if (dl) cudaFree(dl);
+        if (tk) cudaFree(tk);
         return cuda_fail(e, "crp_sim_reserve");
     }
     free_state(s->st);
     cudaFree(s->lists[0]);
     cudaFree(s->lists[1]);
     cudaFree(s->done_list);
+    cudaFree(s->taken);
+    s->taken = tk;
     s->st = ns;
     s->lists[0] = l0;
     s->lists[1] = l1;
@@ -1020,7 +1045,7 @@ extern "C" {
 int crp_kernel_runs(uint64_t* count) {
     if (!count) return fail(CRP_ERR_INVALID_ARG, "count is NULL");
     CRP_CUDA(cudaDeviceSynchronize());
-    *count = kernel_runs_capi() + kernel_runs_fp64() + kernel_runs_mixed() + kernel_runs_adjoint() +
+    *count = kernel_runs_capi() + kernel_runs_fp64() + kernel_runs_team() + kernel_runs_mixed() + kernel_runs_adjoint() +
              kernel_runs_sources() + kernel_runs_lens();
     return CRP_OK;
 }
@@ -1308,10 +1333,11 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
         return fail(CRP_ERR_INVALID_ARG, "the mixed form reads FP32 or BF16 grids");
     const bool mixed = prm->form == CRP_FORM_MIXED;
     const int order = prm->order == CRP_ORDER_DEFAULT ? CRP_ORDER_COST : prm->order;
-    const int pickup = prm->pickup == CRP_PICKUP_DEFAULT ? CRP_PICKUP_OFF : prm->pickup;
+    const int pickup = prm->pickup;
     if (order != CRP_ORDER_SLOT && order != CRP_ORDER_COST && order != CRP_ORDER_GRID)
         return fail(CRP_ERR_INVALID_ARG, "unknown order");
-    if (pickup != CRP_PICKUP_OFF && pickup != CRP_PICKUP_ON) return fail(CRP_ERR_INVALID_ARG, "unknown pickup");
+    if (pickup != CRP_PICKUP_DEFAULT && pickup != CRP_PICKUP_OFF && pickup != CRP_PICKUP_ON)
+        return fail(CRP_ERR_INVALID_ARG, "unknown pickup");
     const int block = prm->block_size > 0 ? prm->block_size : 128;
     if (block % 32 || block > 256) return fail(CRP_ERR_INVALID_ARG, "block_size must be a multiple of 32, <= 256");
     // the FP64 form reads FP64 copies of the grids (no per-corner widening on the FP64 pipe)
@@ -1354,7 +1380,28 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
         if (oe != 0 || occ < 1) occ = 1;
         bps = occ;
     }
-    P.grid = (s->sms > 0 ? s->sms : 1) * bps;
+    const int sms = s->sms > 0 ? s->sms : 1;
+    PropArgs& a = P.a;
+    P.grid = sms * bps;
+    // FP64: the one-lane kernel for what fills its lanes, the three-lane kernel for the rest
+    // (simulations that can't fill them launch only that). PICKUP_ON asks for the one-lane
+    // kernel's own handling of secondaries.
+    const bool team = !mixed && pickup != CRP_PICKUP_ON && layout == LAYOUT_F64X4;
+    const long long lanes = (long long)P.grid * block;
+    // Without tables there are no secondaries and one launch does; with them the second takes those
+    // that the first left (all, if they wait for it).
+    P.team_grid = P.team_block = P.team_launches = 0;
+    P.lane_launches = mixed && !s->tables ? 1 : 2;
+    if (team) {
+        int occ = prm->blocks_per_sm;
+        if (occ <= 0 && (propagate_team_occupancy(s->mod, p2, block, &occ) != 0 || occ < 1)) occ = 1;
+        P.team_grid = sms * occ;
+        P.team_block = block;
+        P.lane_launches = s->capacity <= lanes ? 0 : (s->tables && pickup == CRP_PICKUP_OFF ? 2 : 1);
+        // what one block per SM takes up needs no launch that drains
+        a.drain_at = (long long)sms * (block / 32) * kTeamsPerWarp;
+        P.team_launches = s->capacity <= a.drain_at || !s->tables ? 2 : 3;
+    }
     P.block = block;
     P.order = order;
     P.mixed = mixed ? 1 : 0;
@@ -1362,7 +1409,6 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
     P.mod = s->mod;
     P.p2 = p2;
     P.n_buckets = order == CRP_ORDER_GRID ? kBuckets * (int)s->host_fields.size() : kBuckets;
-    PropArgs& a = P.a;
     a.st = s->st;
     a.fields = fields;
     a.n_fields = (int)s->host_fields.size();
@@ -1375,7 +1421,11 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
     // default cadence: 2 attempts between refill checks in the precision form (measured +1.5 %
     // on the 10^6-nuclei workload), 1 in the FP64 form; results do not depend on it
     a.cadence = prm->cadence > 0 ? prm->cadence : (prm->form == CRP_FORM_MIXED ? 2 : 1);
-    a.pickup = pickup == CRP_PICKUP_ON ? 1 : 0;
+    a.pickup = pickup == CRP_PICKUP_ON ? 1 : (pickup == CRP_PICKUP_DEFAULT && s->tables ? 2 : 0);
+    a.drain = team ? 1 : 0;
+    a.min_work = team ? lanes : -1;
+    a.taken = team ? s->taken : nullptr;
+    a.back = team ? 1 : 0;
     a.lists[0] = s->lists[0];
     a.lists[1] = s->lists[1];
     a.done_list = s->done_list;
@@ -1416,14 +1466,27 @@ int enqueue(crp_sim* s, const Plan& P, cudaStream_t st) {
     CRP_CUDA(cudaGetLastError());
     // generation 1: the work list (and, with pickup, secondaries it pushes once the list
     // runs dry); generation 2: the secondaries left. Nucleon secondaries never split, so two
-    // launches finish the call. The push list starts filled with -1.
-    for (int gen = 0; gen < 2; ++gen) {
-        if (a.pickup) CRP_CUDA(cudaMemsetAsync(s->lists[1 - gen], 0xff, sizeof(int32_t) * s->capacity, st));
-        a.list = gen;
+    // launches finish the call. With the three-lane kernel a one-lane launch hands its active
+    // particles on when its list has run out, to the next list with the secondaries, and the
+    // three-lane launches finish them.
+    for (int gen = 0; gen < P.lane_launches; ++gen) {
         int e = P.mixed ? launch_propagate_mixed(a, P.layout, P.mod, P.p2, P.grid, P.block, st)
                         : launch_propagate_fp64(a, P.layout, P.mod, P.p2, P.grid, P.block, st);
         if (e) return cuda_fail((cudaError_t)e, "propagate kernel launch");
-        k_swap<<<1, 1, 0, st>>>(s->ctr, s->capacity, gen);
+        k_swap<<<1, 1, 0, st>>>(s->ctr, s->capacity, a.min_work);
+        CRP_CUDA(cudaGetLastError());
+    }
+    for (int gen = 0; gen < P.team_launches; ++gen) {
+        // one that drains if the particles may not fit one block per SM, one for what is left, and one
+        // for the secondaries that this released late (nucleons, which release nothing)
+        PropArgs t = a;
+        t.drain = gen == 0 && s->capacity > a.drain_at ? 1 : 0;
+        t.min_work = t.drain ? a.drain_at : -1;
+        if (gen == P.team_launches - 1) t.pickup = 0;
+        int e = launch_propagate_team(t, P.mod, P.p2, t.drain ? P.team_grid : std::max(1, s->sms), P.team_block,
+                                      t.drain ? 0 : 1, st);
+        if (e) return cuda_fail((cudaError_t)e, "propagate kernel launch");
+        k_swap<<<1, 1, 0, st>>>(s->ctr, s->capacity, t.min_work);
         CRP_CUDA(cudaGetLastError());
     }
     return CRP_OK;
@@ -1449,8 +1512,9 @@ __global__ void k_loop_cond(Counters* C, cudaGraphConditionalHandle h, long long
 bool same_plan(const Plan& x, const Plan& y) {
     return std::memcmp(&x.a, &y.a, sizeof(PropArgs)) == 0 && x.grid == y.grid &&
            x.block == y.block && x.order == y.order && x.mixed == y.mixed && x.n_buckets == y.n_buckets &&
-           x.p2 == y.p2 &&
-           x.layout == y.layout;
+           x.p2 == y.p2 && x.team_grid == y.team_grid && x.team_block == y.team_block &&
+           x.team_launches == y.team_launches &&
+           x.lane_launches == y.lane_launches && x.layout == y.layout && x.mod == y.mod;
 }
 
 }  // namespace
@@ -1768,11 +1832,11 @@ extern "C" int crp_propagate_noalloc(const void* grid, int32_t nx, int32_t ny, i
     a.lists[1] = l1;
     a.done_list = done;
     a.ctr = ctr;
+    a.min_work = -1;
     for (int gen = 0; gen < 2; ++gen) {
-        a.list = gen;
         int e = launch_propagate_fp64(a, LAYOUT_F32X4, 0, f.pow2, sms * occ, block, st);
         if (e) return cuda_fail((cudaError_t)e, "propagate kernel launch");
-        k_swap<<<1, 1, 0, st>>>(ctr, n, gen);
+        k_swap<<<1, 1, 0, st>>>(ctr, n, -1);
         CRP_CUDA(cudaGetLastError());
     }
     CRP_CUDA(cudaStreamSynchronize(st));

@@ -94,6 +94,39 @@ __device__ __forceinline__ void floor_split(double r, long long& i, double& fl) 
     }
 }
 
+// The double G 2^-52 for 0 <= G <= 2^52, exactly, with integer instructions.
+__device__ __forceinline__ double fixed52(unsigned long long G) {
+    if (G == 0) return 0.0;
+    const int z = __clzll((long long)G);               // 11 .. 63
+    return __longlong_as_double(((long long)(1034 - z) << 52) + (long long)((G << (z - 11)) & 0xFFFFFFFFFFFFFull));
+}
+
+// floor(r) and the weights w0 = 1 - (r - floor r), w1 = r - floor r, as floor_split and the two FP64
+// subtractions give them. For 1 <= |r| < 2^52 the fraction is a multiple of 2^-52, both weights are
+// exact, and they are formed with integer instructions; elsewhere by the subtractions. Where the
+// FP64 pipe is the limit (the three-lane kernel with full warps: 84 % busy) this takes 6 % off an
+// attempt; the one-lane kernel, with two warps per sub-partition, waits on its instructions in turn
+// and gained nothing from it.
+__device__ __forceinline__ void floor_weights(double r, long long& i, double& w0, double& w1) {
+    const long long b = __double_as_longlong(r);
+    const int ef = (int)((b >> 52) & 0x7FF);
+    if (ef >= 1023 && ef < 1075) {
+        const unsigned long long m = ((unsigned long long)b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+        const long long n = (long long)(m >> (1075 - ef));                                   // |trunc r|
+        const unsigned long long f = (m << (ef - 1023)) & 0xFFFFFFFFFFFFFull;                // |r| - n, in 2^-52
+        const bool neg = b < 0, up = neg && f != 0;                                          // floor = -(n + 1)
+        i = neg ? -(n + (up ? 1 : 0)) : n;
+        const unsigned long long g = up ? 0x10000000000000ull - f : f;
+        w1 = fixed52(g);
+        w0 = fixed52(0x10000000000000ull - g);
+    } else {
+        double fl;
+        floor_split(r, i, fl);
+        w1 = r - fl;
+        w0 = 1.0 - w1;
+    }
+}
+
 // One axis of the periodic lookup: r = x (1/spacing) - o (1/spacing) with one rounding (oi is
 // the product o (1/spacing), rounded once), i0 = floor(r) mod n, weights (1 - f, f). P2: the
 // caller guarantees n is a power of two, and the 64-bit modulo's code (inlined at every
@@ -105,14 +138,20 @@ __device__ __forceinline__ void axis(double x, double oi, double inv, int n, int
     long long i;
     double fl;
     floor_split(r, i, fl);
-    const double fr = r - fl;
+    w1 = r - fl;
+    w0 = 1.0 - w1;
     long long a;
-    if (P2 || pow2) a = i & (long long)(n - 1);
-    else { a = i % n; if (a < 0) a += n; }
+    if (P2 || pow2) {
+        a = i & (long long)(n - 1);
+    } else if (i == (long long)(int)i) {   // the 32-bit remainder is a third of the 64-bit one
+        a = (int)i % n;
+        if (a < 0) a += n;
+    } else {
+        a = i % n;
+        if (a < 0) a += n;
+    }
     i0 = a;
     i1 = (a + 1 == n) ? 0 : a + 1;
-    w0 = 1.0 - fr;
-    w1 = fr;
 }
 
 // Modulation value M(x): scalar periodic trilinear lookup on the modulation grid, corners
@@ -344,6 +383,15 @@ __device__ __forceinline__ float pow2_series(float y) {
 __device__ __forceinline__ float ctrl_factor(float log2r, float p, float lo, float hi) {
     const float y = fminf(fmaxf(__fmul_rn(p, log2r), -8.0f), 8.0f);
     return fminf(fmaxf(__fmul_rn(0.95f, pow2_series(y)), lo), hi);
+}
+
+// The factor of an attempt's size for the next one: shrink (rejected) or growth (accepted; 5 for a
+// zero-length step or a zero error). Both come from one evaluation with selected constants, so that
+// lanes that accept and lanes that retry run it together.
+__device__ __forceinline__ float step_factor(bool accept, double sx, double su, double h, float lg_tol) {
+    const float f = ctrl_factor(ctrl_log2r(sx, su, h, lg_tol), accept ? -0.2f : -0.25f, accept ? 0.2f : 0.1f,
+                                accept ? 5.0f : 1.0f);
+    return accept && (is_zero(h) || (is_zero(sx) && is_zero(su))) ? 5.0f : f;
 }
 
 // Exact widening of a normal float (the clamped factors) to double with integer

@@ -83,7 +83,11 @@ struct Counters {
     unsigned long long slices;       // slices run by the current propagate loop
     unsigned long long prev_accepted;
     unsigned int status_bits;
-    unsigned int pad_;
+    int cur;                         // work list (0 or 1) that the next propagate launch takes
+    int pushed;                      // that list was filled by a propagate launch of this call
+    int pad_;
+    unsigned long long head0;        // first entry of that list (earlier ones were picked up when pushed)
+    unsigned long long left;         // entries of the list whose particle the current launch has stored
 };
 
 struct PropArgs {
@@ -97,9 +101,14 @@ struct PropArgs {
     long long max_steps;
     long long capacity;
     int32_t cadence;
-    int32_t pickup;                  // take secondaries pushed during the launch
-    int32_t list;                    // process list `list`, push secondaries to 1 - list
-    int32_t* lists[2];
+    int32_t pickup;                  // take secondaries pushed during the launch: 1 once the list has run
+                                     // out, 2 before the rest of the list
+    int32_t drain;                   // once the list has run out (and, in the three-lane kernel, at most
+    int32_t back;                    // drain_at particles are left), hand active particles to the next launch
+    long long drain_at;              // back: lists that a launch of this call filled are taken from their end
+    long long min_work;              // a launch leaves lists of at most this many entries to the next one
+    int32_t* taken;                  // per slot: accepted steps of this call so far (drained particles); may be NULL
+    int32_t* lists[2];               // list Counters::cur is processed, secondaries are pushed to the other
     int32_t* done_list;
     Counters* ctr;
     // reflective box (boundary = 1): per axis origin, origin + size, size, 1/size
@@ -127,6 +136,10 @@ int launch_lens_bin(const SimState& S, const Counters* C, int nside, int n_mat, 
 // indices with a mask; with p2 = 0 they take the general wrap, valid for any size).
 int launch_propagate_fp64(const PropArgs& a, int layout, int mod, int p2, int grid, int block, void* stream);
 int propagate_fp64_occupancy(int layout, int mod, int p2, int block, int* blocks_per_sm);
+// Three lanes per particle (propagate_team.cu); reads FP64 node copies only.
+constexpr int kTeamsPerWarp = 10;
+int launch_propagate_team(const PropArgs& a, int mod, int p2, int grid, int block, int one_per_sm, void* stream);
+int propagate_team_occupancy(int mod, int p2, int block, int* blocks_per_sm);
 int launch_propagate_mixed(const PropArgs& a, int layout, int mod, int p2, int grid, int block, void* stream);
 int propagate_mixed_occupancy(int layout, int mod, int p2, int block, int* blocks_per_sm);
 
@@ -139,6 +152,7 @@ int propagate_mixed_occupancy(int layout, int mod, int p2, int block, int* block
     } while (0)
 unsigned long long kernel_runs_capi();
 unsigned long long kernel_runs_fp64();
+unsigned long long kernel_runs_team();
 unsigned long long kernel_runs_mixed();
 unsigned long long kernel_runs_adjoint();
 unsigned long long kernel_runs_sources();

@@ -20,75 +20,129 @@ __device__ __forceinline__ unsigned long long ld_volatile(const unsigned long lo
     return *(volatile const unsigned long long*)p;
 }
 
-// Waits, at most `limit` times 64 ns, for a non-negative value to be published at p (acquire
+// Waits, at most `limit` times 64 ns, for a value other than -1 to be published at p (acquire
 // loads). Returns false if it never appeared; the caller turns that into a status bit.
 __device__ __forceinline__ bool bounded_acquire_wait(int32_t* p, int limit, int32_t& v) {
     cuda::atomic_ref<int32_t, cuda::thread_scope_device> e(*p);
     for (int t = 0; t < limit; ++t) {
         v = e.load(cuda::memory_order_acquire);
-        if (v >= 0) return true;
+        if (v != -1) return true;
         __nanosleep(64);
     }
     return false;
 }
 
-// Append slot q to the list the launch pushes into (secondaries).
-__device__ __forceinline__ void sched_push(const PropArgs& a, int32_t q) {
-    const int L = 1 - a.list;
+// Append entry q to work list L.
+__device__ __forceinline__ void sched_push(const PropArgs& a, int L, int32_t q) {
     const unsigned long long p = atomicAdd(&a.ctr->count[L], 1ull);
     cuda::atomic_ref<int32_t, cuda::thread_scope_device> e(a.lists[L][p]);
     e.store(q, cuda::memory_order_release);
 }
 
-// Returns the slot this lane should load next, or -1. Lanes with idle == false get -1.
-__device__ __forceinline__ int sched_pop(const PropArgs& a, bool idle, int lane,
-                                        unsigned long long n_work, unsigned& bits) {
+// Entries of a work list: the slot of a particle, or kResumed - slot for one that the previous launch
+// of the call handed on; -1: not yet published. Whoever takes an entry leaves -1, so that the lists of
+// a simulation hold nothing else between calls and need no clearing before a launch pushes.
+constexpr int32_t kResumed = -2;
+
+__device__ __forceinline__ int sched_slot(const PropArgs& a, int32_t v, unsigned& bits, int& resumed) {
+    if (v <= kResumed && a.taken) {
+        v = kResumed - v;
+        resumed = 1;
+    }
+    if (v < 0 || v >= a.capacity) { bits |= BIT_BOUNDS; return -1; }
+    return v;
+}
+
+// What a launch works through: list L from position head0 (entries before it were taken by the
+// previous launch) to n_work. back: from the end (a list that a launch filled ends with the
+// particles handed on, the long ones).
+struct WorkList {
+    int L;
+    bool back;
+    unsigned long long n_work, head0;
+};
+__device__ __forceinline__ WorkList work_list(const PropArgs& a) {
+    const Counters* C = a.ctr;
+    const int L = *(volatile const int*)&C->cur;
+    return {L, a.back && *(volatile const int*)&C->pushed, ld_volatile(&C->count[L]), ld_volatile(&C->head0)};
+}
+
+// Returns the slot this lane should load next from the work list, or -1. Lanes with idle == false
+// get -1. dry (the same in all lanes) turns true once the list has run out for good.
+__device__ __forceinline__ int sched_pop(const PropArgs& a, const WorkList& W, bool idle, int lane, unsigned& bits,
+                                        bool& dry, int& resumed) {
     const unsigned im = __ballot_sync(kSchedFull, idle);
     if (!im) return -1;
     Counters* C = a.ctr;
-    const int L = a.list, P = 1 - a.list;
     unsigned long long base = 0;
-    unsigned got = 0, from = 0;
+    unsigned got = 0, out = 0;
     if (lane == 0) {
         const unsigned need = (unsigned)__popc(im);
-        if (ld_volatile(&C->head[L]) < n_work) {
-            base = atomicAdd(&C->head[L], (unsigned long long)need);
-            if (base < n_work) got = (unsigned)min((unsigned long long)need, n_work - base);
+        if (ld_volatile(&C->head[W.L]) < W.n_work) {
+            base = atomicAdd(&C->head[W.L], (unsigned long long)need);
+            if (base < W.n_work) got = (unsigned)min((unsigned long long)need, W.n_work - base);
         }
-        if (got == 0 && a.pickup) {   // secondaries pushed so far in this launch
-            from = 1;
-            for (int t = 0; t < kClaimRetryLimit; ++t) {
-                const unsigned long long h = ld_volatile(&C->head[P]);
-                const unsigned long long c = ld_volatile(&C->count[P]);
-                if (h >= c) break;
-                const unsigned take = (unsigned)min((unsigned long long)need, c - h);
-                if (atomicCAS(&C->head[P], h, h + take) == h) {
-                    base = h;
-                    got = take;
-                    break;
-                }
+        out = got < need;
+    }
+    base = __shfl_sync(kSchedFull, base, 0);
+    got = __shfl_sync(kSchedFull, got, 0);
+    dry = __shfl_sync(kSchedFull, out, 0);
+    if (!idle) return -1;
+    const unsigned rank = (unsigned)__popc(im & ((1u << lane) - 1u));
+    if (rank >= got) return -1;
+    const unsigned long long pos = base + rank;
+    int32_t* e = a.lists[W.L] + (W.back ? W.n_work - 1 - (pos - W.head0) : pos);
+    const int32_t v = *e;
+    *e = -1;
+    return sched_slot(a, v, bits, resumed);
+}
+
+// Whether idle lanes look for pushed secondaries in this turn of the one-lane kernels: now and then
+// while the list lasts, seldom once it has run out. The look is a round trip to L2, and with thousands
+// of warps asking it is the counters' line that everyone waits for (10^6 nuclei in the precision form:
+// 73 ms without pick-ups; 265, 114, 81, 66 ms looking every 1, 4, 16, 64 turns; 68 ms every 16 and, with
+// the list empty, every 128. 10^5 nuclei in the modulated scenario: 65 ms without, 44 to 47 ms with).
+// The FP64 form, whose turns take ten times as long, looks every 4 (200 000 nuclei: 284 ms without,
+// 247 ms, 267 ms looking every 32).
+template <unsigned Every>
+__device__ __forceinline__ bool sched_look(const PropArgs& a, bool dry, unsigned turn) {
+    return a.pickup && (dry ? turn % 128 == 0 : (a.pickup == 2 && turn % Every == 0));
+}
+
+// The same from list P, into which this launch pushes: claims positions below the push count and
+// waits, bounded, for the entries to be published.
+__device__ __forceinline__ int sched_pick(const PropArgs& a, int P, bool idle, int lane, unsigned& bits, int& resumed) {
+    const unsigned im = __ballot_sync(kSchedFull, idle);
+    if (!im) return -1;
+    Counters* C = a.ctr;
+    unsigned long long base = 0;
+    unsigned got = 0;
+    if (lane == 0) {
+        const unsigned need = (unsigned)__popc(im);
+        for (int t = 0; t < kClaimRetryLimit; ++t) {
+            const unsigned long long h = ld_volatile(&C->head[P]);
+            const unsigned long long c = ld_volatile(&C->count[P]);
+            if (h >= c) break;
+            const unsigned take = (unsigned)min((unsigned long long)need, c - h);
+            if (atomicCAS(&C->head[P], h, h + take) == h) {
+                base = h;
+                got = take;
+                break;
             }
         }
     }
     base = __shfl_sync(kSchedFull, base, 0);
     got = __shfl_sync(kSchedFull, got, 0);
-    from = __shfl_sync(kSchedFull, from, 0);
     if (!idle) return -1;
     const unsigned rank = (unsigned)__popc(im & ((1u << lane) - 1u));
     if (rank >= got) return -1;
-    const unsigned long long pos = base + rank;
-    if (from == 0) {
-        const int32_t v = a.lists[L][pos];
-        if (v < 0 || v >= a.capacity) { bits |= BIT_BOUNDS; return -1; }
-        return v;
-    }
     int32_t v = -1;
-    if (!bounded_acquire_wait(a.lists[P] + pos, kPublishWaitLimit, v)) {
+    if (!bounded_acquire_wait(a.lists[P] + base + rank, kPublishWaitLimit, v)) {
         bits |= BIT_TIMEOUT;   // the entry never appeared: reported by crp_sync
         return -1;
     }
-    if (v >= a.capacity) { bits |= BIT_BOUNDS; return -1; }
-    return v;
+    a.lists[P][base + rank] = -1;
+    return sched_slot(a, v, bits, resumed);
 }
 
 }  // namespace crp

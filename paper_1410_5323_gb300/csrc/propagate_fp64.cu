@@ -5,8 +5,10 @@
 // one loop iteration is one Cash-Karp attempt, so lanes that reject and lanes that start
 // a new step stay converged. Idle lanes are refilled from a global work counter with one
 // warp-aggregated atomic (ballot + popc); finished particles are appended to the done
-// list; secondaries reserve a slot atomically and go to the other work list, which a
-// second launch of this kernel processes.
+// list; secondaries reserve a slot atomically and go to the other work list, from which
+// idle lanes of this launch or the next launch take them. When the work list has run out
+// the particles still active go to the other list too, for the kernel that has three lanes
+// per particle (propagate_team.cu): a trajectory's time here is 23 us an attempt at the least.
 //
 // Compiled with --fmad=false: every FP64 expression is evaluated as written, in the same
 // order as the stated reading, so results are bit-identical to the FP64 oracle. Work that
@@ -47,7 +49,9 @@ __global__ void CRP_FP64_BOUNDS k_propagate_fp64(const PropArgs a) {
     CRP_COUNT_RUN();
     const int lane = threadIdx.x & 31;
     Counters* C = a.ctr;
-    const unsigned long long n_work = *(volatile unsigned long long*)&C->count[a.list];
+    const WorkList work = work_list(a);
+    const int pushes = 1 - work.L;
+    if ((long long)(work.n_work - work.head0) <= a.min_work) return;
     const double INF = __longlong_as_double(0x7ff0000000000000LL);
     const SimState& S = a.st;
 
@@ -80,10 +84,27 @@ __global__ void CRP_FP64_BOUNDS k_propagate_fp64(const PropArgs a) {
         slot = -1;
     };
 
-    for (;;) {
+    bool dry = false;
+    for (unsigned turn = 0;; ++turn) {
         // ---- refill idle lanes from the work list (one atomic per warp) ----
-        const bool idle = slot < 0;
-        const int popped = sched_pop(a, idle, lane, n_work, bits);
+        int popped = -1, resumed = 0;
+        if (sched_look<4>(a, dry, turn) && !(dry && a.drain))
+            popped = sched_pick(a, pushes, slot < 0, lane, bits, resumed);
+        if (!dry) {
+            const int p = sched_pop(a, work, slot < 0 && popped < 0, lane, bits, dry, resumed);
+            if (p >= 0) popped = p;
+            if (a.drain && turn % 8 == 7) {   // a full warp asks for nothing: look whether the list has run out
+                unsigned long long head = lane == 0 ? ld_volatile(&C->head[work.L]) : 0ull;
+                head = __shfl_sync(kFull, head, 0);
+                dry = dry || head >= work.n_work;
+            }
+        }
+        if (a.drain && dry && popped < 0 && slot >= 0 && new_step) {   // the next launch resumes it here
+            const int32_t q = slot;
+            a.taken[q] = (int32_t)taken;
+            store(CRP_STATUS_ACTIVE_);
+            sched_push(a, pushes, kResumed - q);
+        }
         if (popped >= 0) {
             slot = popped;
             y.x = __ldcg(&S.x[slot]); y.y = __ldcg(&S.y[slot]); y.z = __ldcg(&S.z[slot]);
@@ -92,7 +113,7 @@ __global__ void CRP_FP64_BOUNDS k_propagate_fp64(const PropArgs a) {
             A = __ldcg(&S.A[slot]); Z = __ldcg(&S.Z[slot]); n_int = __ldcg(&S.n_int[slot]); gid = __ldcg(&S.grid_id[slot]);
             uid = (unsigned long long)__ldcg(&S.uid[slot]);
             n_steps = __ldcg(&S.n_steps[slot]); n_att = __ldcg(&S.n_att[slot]);
-            taken = 0;
+            taken = resumed ? __ldcg(&a.taken[slot]) : 0;
             new_step = true;
             if (gid < 0 || gid >= a.n_fields) { bits |= BIT_BOUNDS; slot = -1; }
         }
@@ -133,9 +154,10 @@ __global__ void CRP_FP64_BOUNDS k_propagate_fp64(const PropArgs a) {
             att_step += 1;
             double sx, su;
             error_sums(err, sx, su);
-            if (!(error_accept(sx, su, h, a.tol, tol2) || le_pos(h, a.hmin))) {
-                const float shrink = ctrl_factor(ctrl_log2r(sx, su, h, lg_tol), -0.25f, 0.1f, 1.0f);
-                h = max_pos(h * widen_normal(shrink), a.hmin);
+            const bool accept = error_accept(sx, su, h, a.tol, tol2) || le_pos(h, a.hmin);
+            const double hnew = h * widen_normal(step_factor(accept, sx, su, h, lg_tol));
+            if (!accept) {
+                h = max_pos(hnew, a.hmin);
                 rejected = 1;
                 continue;
             }
@@ -176,9 +198,7 @@ __global__ void CRP_FP64_BOUNDS k_propagate_fp64(const PropArgs a) {
             n_steps += 1;
             acc_tot += 1;
             taken += 1;
-            const float grow = (is_zero(h) || (is_zero(sx) && is_zero(su)))
-                                   ? 5.0f : ctrl_factor(ctrl_log2r(sx, su, h, lg_tol), -0.2f, 0.2f, 5.0f);
-            double hnext = h * widen_normal(grow);
+            double hnext = hnew;
             if (!rejected && lt_pos(h_first, h_propc)) hnext = max_pos(hnext, h_propc);
             hprop = clampd(hnext, a.hmin, a.hmax);
             // ---- continuous loss at gamma0 ----
@@ -206,7 +226,7 @@ __global__ void CRP_FP64_BOUNDS k_propagate_fp64(const PropArgs a) {
                         const unsigned long long d = atomicAdd(&C->n_done, 1ull);
                         a.done_list[d] = (int32_t)qs;
                     } else {
-                        sched_push(a, (int32_t)qs);
+                        sched_push(a, pushes, (int32_t)qs);
                     }
                     sec_tot += 1;
                     A = A - 1;

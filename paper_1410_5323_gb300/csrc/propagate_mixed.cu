@@ -344,7 +344,8 @@ template <int L, bool M, bool P2>
 __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* sm) {
     const int lane = threadIdx.x & 31;
     Counters* C = a.ctr;
-    const unsigned long long n_work = *(volatile unsigned long long*)&C->count[a.list];
+    const WorkList work = work_list(a);
+    const int pushes = 1 - work.L;
     const float INF = __int_as_float(0x7f800000);
     const SimState& S = a.st;
     const double tol2 = a.tol * a.tol;
@@ -411,9 +412,14 @@ __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* s
         slot = -1;
     };
 
-    for (;;) {
-        const bool idle = slot < 0;
-        const int popped = sched_pop(a, idle, lane, n_work, bits);
+    bool dry = false;
+    for (unsigned turn = 0;; ++turn) {
+        int popped = -1, resumed = 0;
+        if (sched_look<32>(a, dry, turn)) popped = sched_pick(a, pushes, slot < 0, lane, bits, resumed);
+        if (!dry) {
+            const int p = sched_pop(a, work, slot < 0 && popped < 0, lane, bits, dry, resumed);
+            if (p >= 0) popped = p;
+        }
         if (popped >= 0) {
             slot = popped;
             gid = __ldcg(&S.grid_id[slot]);
@@ -678,7 +684,7 @@ __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* s
                         const unsigned long long d = atomicAdd(&C->n_done, 1ull);
                         a.done_list[d] = (int32_t)qs;
                     } else {
-                        sched_push(a, (int32_t)qs);
+                        sched_push(a, pushes, (int32_t)qs);
                     }
                     sec_tot += 1;
                     A = A - 1;

@@ -1,0 +1,78 @@
+"""The three-lane FP64 kernel and the hand-over between the propagate kernels of a call: batches
+around the sizes of a team, a warp and one block per SM, batches above the one-lane kernel's lanes
+(which pass through every launch), secondaries taken up while they come, budgets that span a
+hand-over, and each option of the path, bit for bit against the oracle."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1410_5323_gb300 import inputs as I
+from _parity import assert_bit_identical, by_uid, run_gpu, run_oracle
+
+pytestmark = pytest.mark.gpu
+MIX = (("H", .4), ("He", .3), ("N", .2), ("Fe", .1))
+
+
+def _grid(n, seed):
+    return I.kolmogorov_grid(n, 0.25 * I.MPC, 2, 8, 1e-13, seed).astype(np.float32)
+
+
+def _same(*args, **kw):
+    sim, rc = run_gpu(*args, **kw)
+    assert rc == 0
+    st, orc = run_oracle(*args, **kw)
+    assert orc == 0
+    assert_bit_identical(sim.state(), st.snapshot())
+    return sim
+
+
+@pytest.mark.parametrize("n", [1, 2, 10, 11, 6081])
+def test_batches_around_a_warp_and_a_layer(oracle_lib, n):
+    p = I.make_particles(n, n, species=MIX, energy=("power", 1e18, 10 ** 20.5, 2.0))
+    _same([_grid(16, 5)], p, I.constant_rate_tables(1 / (200 * I.MPC), 1 / (8 * I.MPC)), 1e-4, I.KPC, I.MPC, 3 * I.MPC,
+          seed=n, capacity=56 * n)
+
+
+@pytest.mark.parametrize("max_steps,calls", [(0, 1), (4, 6)])
+def test_batches_above_the_one_lane_kernels_lanes(oracle_lib, max_steps, calls):
+    """60 000 nuclei that interact every few steps: one-lane launches, both three-lane launches, and
+    budgets whose count goes with a particle that is handed on."""
+    n = 60_000
+    p = I.make_particles(n, 3, species=MIX, energy=("power", 3e18, 10 ** 20.5, 2.0))
+    sim = _same([_grid(16, 6)], p, I.constant_rate_tables(0.0, 1 / (3 * I.MPC)), 1e-4, I.KPC, I.MPC, 2 * I.MPC, seed=9,
+                capacity=6 * n, max_steps=max_steps, calls=calls)
+    assert sim.counts()["secondaries"] > n // 10
+
+
+@pytest.mark.parametrize("pickup", [0, 1, 2])
+def test_pickup_modes_give_the_same_particles(pickup):
+    import paper_1410_5323_gb300 as crp
+
+    p = I.make_particles(2000, 8, species=MIX, energy=("power", 1e18, 10 ** 20.5, 2.0))
+    f, t = crp.Field(_grid(16, 7), 0.25 * I.MPC), crp.Tables(I.constant_rate_tables(1 / (300 * I.MPC), 1 / (4 * I.MPC)))
+    states = []
+    for form in (crp.FORM_FP64, crp.FORM_MIXED):
+        for mode in (1, pickup):
+            sim = crp.Simulation([f], t, seed=2, capacity=56 * 2000)
+            sim.inject(p)
+            sim.propagate(1e-4, I.KPC, I.MPC, 8 * I.MPC, form=form, pickup=mode)
+            assert sim.sync(60.0) == 0
+            states.append(by_uid(sim.state()))
+    for a, b in ((0, 1), (2, 3)):
+        for k in states[a]:
+            assert np.array_equal(states[a][k], states[b][k], equal_nan=states[a][k].dtype.kind == "f"), k
+
+
+def test_options_small_batch(oracle_lib):
+    """Non-power-of-two grids with an origin and negative coordinates, a modulation grid, a reflective
+    box, two fields of different realisations."""
+    n = 83
+    rng = np.random.default_rng(4)
+    p = I.make_particles(n, 12, species=(("H", .5), ("Fe", .5)), energy=("power", 1e18, 1e20, 2.0))
+    box = ((-2 * I.MPC, -1.5 * I.MPC, 0.0), (4 * I.MPC, 5 * I.MPC, 4.5 * I.MPC))
+    p.x[:] = np.asarray(box[0]) + rng.uniform(0.1, 0.9, (n, 3)) * np.asarray(box[1])
+    p.grid_id[:] = np.arange(n) % 2
+    mods = [np.exp(rng.normal(0.0, 0.4, (6, 5, 7))).astype(np.float32) for _ in range(2)]
+    grids = [_grid(18, 13), _grid(18, 14)]
+    _same(grids, p, None, 1e-4, I.KPC, I.MPC, 6 * I.MPC, origin=(0.3 * I.MPC, -0.1 * I.MPC, 0.0), mods=mods,
+          mod_spacing=0.6 * I.MPC, box=box)
