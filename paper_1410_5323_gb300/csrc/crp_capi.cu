@@ -332,11 +332,21 @@ __global__ void k_build_worklist(const int32_t* __restrict__ status, int32_t* __
 
 // After a propagate launch over list C->cur: fix the slot count, reset the pop head and the list
 // that the next launch pushes into, and make the other list the next one. A one-lane launch that
-// left its list alone (at most min_work entries) changes nothing.
-__global__ void k_swap(Counters* C, long long capacity, long long min_work) {
+// left its list alone (at most min_work entries) changes nothing. One block; in calls that take
+// secondaries up (l0 not NULL) it puts -1 back into the list, whose entries would otherwise pass for
+// published ones when a launch pushes into it. (Left to whoever takes an entry, that store slowed the
+// launch: 10^6 sources of a sky map 1.8 -> 2.5 ms, 10^6 nuclei 68 -> 73 ms.)
+__global__ void k_swap(Counters* C, long long capacity, long long min_work, int32_t* l0, int32_t* l1) {
     CRP_COUNT_RUN();
     const int from = C->cur;
-    if ((long long)(C->count[from] - C->head0) <= min_work) return;
+    const long long n = (long long)C->count[from];
+    if (n - (long long)C->head0 <= min_work) return;
+    if (l0) {
+        int32_t* l = from ? l1 : l0;
+        for (long long i = threadIdx.x; i < n; i += blockDim.x) l[i] = -1;
+    }
+    __syncthreads();
+    if (threadIdx.x) return;
     const unsigned long long r = C->reserve;
     C->n_used = r < (unsigned long long)capacity ? r : (unsigned long long)capacity;
     C->reserve = C->n_used;
@@ -463,6 +473,7 @@ struct crp_sim {
     int32_t* lists[2] = {nullptr, nullptr};
     int32_t* done_list = nullptr;
     Counters* ctr = nullptr;
+    bool untidy = false;                // the work lists may hold entries of an earlier call
     int32_t* taken = nullptr;           // accepted steps of this call, for particles handed between launches
     unsigned* sort_scratch = nullptr;   // [hist n_buckets][offsets n_buckets]
     cudaStream_t last = nullptr;
@@ -850,6 +861,7 @@ int crp_sim_reserve(crp_sim* s, int64_t capacity) {
     cudaFree(s->done_list);
     cudaFree(s->taken);
     s->taken = tk;
+    s->untidy = false;
     s->st = ns;
     s->lists[0] = l0;
     s->lists[1] = l1;
@@ -1372,10 +1384,11 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
     }
     int p2 = 1;   // the mask-wrap kernels when every vector grid's sizes are powers of two
     for (const FieldDev& hf : s->host_fields) p2 &= hf.pow2 ? 1 : 0;
+    const int take_up = pickup == CRP_PICKUP_ON ? 1 : (pickup == CRP_PICKUP_DEFAULT && s->tables ? 2 : 0);
     int bps = prm->blocks_per_sm;
     if (bps <= 0) {
         int occ = 0;
-        const int oe = mixed ? propagate_mixed_occupancy(layout, s->mod, p2, block, &occ)
+        const int oe = mixed ? propagate_mixed_occupancy(layout, s->mod, p2, take_up, block, &occ)
                              : propagate_fp64_occupancy(layout, s->mod, p2, block, &occ);
         if (oe != 0 || occ < 1) occ = 1;
         bps = occ;
@@ -1421,7 +1434,7 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
     // default cadence: 2 attempts between refill checks in the precision form (measured +1.5 %
     // on the 10^6-nuclei workload), 1 in the FP64 form; results do not depend on it
     a.cadence = prm->cadence > 0 ? prm->cadence : (prm->form == CRP_FORM_MIXED ? 2 : 1);
-    a.pickup = pickup == CRP_PICKUP_ON ? 1 : (pickup == CRP_PICKUP_DEFAULT && s->tables ? 2 : 0);
+    a.pickup = take_up;
     a.drain = team ? 1 : 0;
     a.min_work = team ? lanes : -1;
     a.taken = team ? s->taken : nullptr;
@@ -1469,11 +1482,12 @@ int enqueue(crp_sim* s, const Plan& P, cudaStream_t st) {
     // launches finish the call. With the three-lane kernel a one-lane launch hands its active
     // particles on when its list has run out, to the next list with the secondaries, and the
     // three-lane launches finish them.
+    const bool tidy = a.pickup != 0;
     for (int gen = 0; gen < P.lane_launches; ++gen) {
         int e = P.mixed ? launch_propagate_mixed(a, P.layout, P.mod, P.p2, P.grid, P.block, st)
                         : launch_propagate_fp64(a, P.layout, P.mod, P.p2, P.grid, P.block, st);
         if (e) return cuda_fail((cudaError_t)e, "propagate kernel launch");
-        k_swap<<<1, 1, 0, st>>>(s->ctr, s->capacity, a.min_work);
+        k_swap<<<1, tidy ? 1024 : 1, 0, st>>>(s->ctr, s->capacity, a.min_work, tidy ? s->lists[0] : nullptr, s->lists[1]);
         CRP_CUDA(cudaGetLastError());
     }
     for (int gen = 0; gen < P.team_launches; ++gen) {
@@ -1486,9 +1500,21 @@ int enqueue(crp_sim* s, const Plan& P, cudaStream_t st) {
         int e = launch_propagate_team(t, P.mod, P.p2, t.drain ? P.team_grid : std::max(1, s->sms), P.team_block,
                                       t.drain ? 0 : 1, st);
         if (e) return cuda_fail((cudaError_t)e, "propagate kernel launch");
-        k_swap<<<1, 1, 0, st>>>(s->ctr, s->capacity, t.min_work);
+        k_swap<<<1, tidy ? 1024 : 1, 0, st>>>(s->ctr, s->capacity, t.min_work, tidy ? s->lists[0] : nullptr, s->lists[1]);
         CRP_CUDA(cudaGetLastError());
     }
+    return CRP_OK;
+}
+
+// Before a call's launches on `st`: clears lists that a call without pick-ups left as they were.
+int tidy_lists(crp_sim* s, const Plan& P, cudaStream_t st) {
+    if (!P.a.pickup) {
+        s->untidy = true;
+        return CRP_OK;
+    }
+    for (int k = 0; k < 2 && s->untidy; ++k)
+        CRP_CUDA(cudaMemsetAsync(s->lists[k], 0xff, sizeof(int32_t) * s->capacity, st));
+    s->untidy = false;
     return CRP_OK;
 }
 
@@ -1528,7 +1554,8 @@ int crp_propagate(crp_sim* s, const crp_params* prm, double tol, double hmin, do
     int rc = make_plan(s, prm, tol, hmin, hmax, dmax, P);
     if (rc) return rc;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    rc = enqueue(s, P, st);
+    rc = tidy_lists(s, P, st);
+    if (!rc) rc = enqueue(s, P, st);
     if (rc) return rc;
     s->last = st;
     return CRP_OK;
@@ -1584,6 +1611,8 @@ int crp_propagate_loop(crp_sim* s, const crp_params* prm, double tol, double hmi
         s->loop_plan = P;
         s->loop_max_slices = max_slices;
     }
+    rc = tidy_lists(s, P, st);
+    if (rc) return rc;
     CRP_CUDA(cudaGraphLaunch(s->loop_exec, st));
     s->last = st;
     return CRP_OK;
@@ -1836,7 +1865,7 @@ extern "C" int crp_propagate_noalloc(const void* grid, int32_t nx, int32_t ny, i
     for (int gen = 0; gen < 2; ++gen) {
         int e = launch_propagate_fp64(a, LAYOUT_F32X4, 0, f.pow2, sms * occ, block, st);
         if (e) return cuda_fail((cudaError_t)e, "propagate kernel launch");
-        k_swap<<<1, 1, 0, st>>>(ctr, n, -1);
+        k_swap<<<1, 1, 0, st>>>(ctr, n, -1, nullptr, nullptr);
         CRP_CUDA(cudaGetLastError());
     }
     CRP_CUDA(cudaStreamSynchronize(st));

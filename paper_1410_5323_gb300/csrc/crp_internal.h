@@ -141,7 +141,7 @@ constexpr int kTeamsPerWarp = 10;
 int launch_propagate_team(const PropArgs& a, int mod, int p2, int grid, int block, int one_per_sm, void* stream);
 int propagate_team_occupancy(int mod, int p2, int block, int* blocks_per_sm);
 int launch_propagate_mixed(const PropArgs& a, int layout, int mod, int p2, int grid, int block, void* stream);
-int propagate_mixed_occupancy(int layout, int mod, int p2, int block, int* blocks_per_sm);
+int propagate_mixed_occupancy(int layout, int mod, int p2, int pick, int block, int* blocks_per_sm);
 
 // Diagnostics: every kernel counts its runs in a device counter of its own translation unit
 // (one atomic per launch, by the first thread of the first block); kernel_runs_*() read them.

@@ -24,6 +24,7 @@ __device__ __forceinline__ unsigned long long ld_volatile(const unsigned long lo
 // loads). Returns false if it never appeared; the caller turns that into a status bit.
 __device__ __forceinline__ bool bounded_acquire_wait(int32_t* p, int limit, int32_t& v) {
     cuda::atomic_ref<int32_t, cuda::thread_scope_device> e(*p);
+#pragma unroll 1
     for (int t = 0; t < limit; ++t) {
         v = e.load(cuda::memory_order_acquire);
         if (v != -1) return true;
@@ -40,8 +41,7 @@ __device__ __forceinline__ void sched_push(const PropArgs& a, int L, int32_t q) 
 }
 
 // Entries of a work list: the slot of a particle, or kResumed - slot for one that the previous launch
-// of the call handed on; -1: not yet published. Whoever takes an entry leaves -1, so that the lists of
-// a simulation hold nothing else between calls and need no clearing before a launch pushes.
+// of the call handed on; -1: not yet published (the bookkeeping after each launch puts it back).
 constexpr int32_t kResumed = -2;
 
 __device__ __forceinline__ int sched_slot(const PropArgs& a, int32_t v, unsigned& bits, int& resumed) {
@@ -91,10 +91,7 @@ __device__ __forceinline__ int sched_pop(const PropArgs& a, const WorkList& W, b
     const unsigned rank = (unsigned)__popc(im & ((1u << lane) - 1u));
     if (rank >= got) return -1;
     const unsigned long long pos = base + rank;
-    int32_t* e = a.lists[W.L] + (W.back ? W.n_work - 1 - (pos - W.head0) : pos);
-    const int32_t v = *e;
-    *e = -1;
-    return sched_slot(a, v, bits, resumed);
+    return sched_slot(a, a.lists[W.L][W.back ? W.n_work - 1 - (pos - W.head0) : pos], bits, resumed);
 }
 
 // Whether idle lanes look for pushed secondaries in this turn of the one-lane kernels: now and then
@@ -119,6 +116,7 @@ __device__ __forceinline__ int sched_pick(const PropArgs& a, int P, bool idle, i
     unsigned got = 0;
     if (lane == 0) {
         const unsigned need = (unsigned)__popc(im);
+#pragma unroll 1
         for (int t = 0; t < kClaimRetryLimit; ++t) {
             const unsigned long long h = ld_volatile(&C->head[P]);
             const unsigned long long c = ld_volatile(&C->count[P]);
@@ -141,7 +139,6 @@ __device__ __forceinline__ int sched_pick(const PropArgs& a, int P, bool idle, i
         bits |= BIT_TIMEOUT;   // the entry never appeared: reported by crp_sync
         return -1;
     }
-    a.lists[P][base + rank] = -1;
     return sched_slot(a, v, bits, resumed);
 }
 

@@ -340,7 +340,9 @@ __device__ __forceinline__ float powf_pos(float r2, float p) { return exp2f(p * 
 
 __device__ __forceinline__ bool fin3(F3 a) { return isfinite(a.x) && isfinite(a.y) && isfinite(a.z); }
 
-template <int L, bool M, bool P2>
+// PICK: idle lanes may take secondaries up (the code for it, though not run without tables, cost runs
+// without them 15 to 30 %: 1024 protons on 64^3 over 100 Mpc 0.93 ms with it, 0.77 ms without).
+template <int L, bool M, bool P2, bool PICK>
 __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* sm) {
     const int lane = threadIdx.x & 31;
     Counters* C = a.ctr;
@@ -415,7 +417,7 @@ __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* s
     bool dry = false;
     for (unsigned turn = 0;; ++turn) {
         int popped = -1, resumed = 0;
-        if (sched_look<32>(a, dry, turn)) popped = sched_pick(a, pushes, slot < 0, lane, bits, resumed);
+        if (PICK && sched_look<32>(a, dry, turn)) popped = sched_pick(a, pushes, slot < 0, lane, bits, resumed);
         if (!dry) {
             const int p = sched_pop(a, work, slot < 0 && popped < 0, lane, bits, dry, resumed);
             if (p >= 0) popped = p;
@@ -737,42 +739,48 @@ __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* s
 
 // Dynamic shared memory: kFieldWords words per thread (field constants), + kModSlots floats per
 // thread for modulated fields.
-template <int L, bool P2>
+template <int L, bool P2, bool PICK>
 __global__ void CRP_MIXED_BOUNDS k_propagate_mixed(const PropArgs a) {
     CRP_COUNT_RUN();
     extern __shared__ double field_sm[];
-    propagate_mixed_body<L, false, P2>(a, reinterpret_cast<float*>(field_sm));
+    propagate_mixed_body<L, false, P2, PICK>(a, reinterpret_cast<float*>(field_sm));
 }
 
-template <int L, bool P2>
+template <int L, bool P2, bool PICK>
 __global__ void CRP_MIXED_MOD_BOUNDS k_propagate_mixed_mod(const PropArgs a) {
     CRP_COUNT_RUN();
     extern __shared__ double mod_sm[];
-    propagate_mixed_body<L, true, P2>(a, reinterpret_cast<float*>(mod_sm));
+    propagate_mixed_body<L, true, P2, PICK>(a, reinterpret_cast<float*>(mod_sm));
 }
 
 }  // namespace
 
-// Kernel for (layout, modulated, power-of-two vector grids): FP32 or BF16 vector grids,
-// node- or cell-major.
+// Kernel for (layout, modulated, power-of-two vector grids, secondaries to take up): FP32 or BF16
+// vector grids, node- or cell-major (the node layouts, read when the cell-major copies found no
+// room, have one kernel for runs with and without secondaries).
+template <int L, bool P2, bool PICK, typename Fn>
+int with_mixed_kernel_of(int mod, Fn&& fn) {
+    return mod ? fn(k_propagate_mixed_mod<L, P2, PICK>) : fn(k_propagate_mixed<L, P2, PICK>);
+}
+
 template <bool P2, typename Fn>
-int with_mixed_kernel_p2(int layout, int mod, Fn&& fn) {
+int with_mixed_kernel_p2(int layout, int mod, int pick, Fn&& fn) {
     switch (layout) {
-    case LAYOUT_F32X4:
-        return mod ? fn(k_propagate_mixed_mod<LAYOUT_F32X4, P2>) : fn(k_propagate_mixed<LAYOUT_F32X4, P2>);
-    case LAYOUT_BF16X4:
-        return mod ? fn(k_propagate_mixed_mod<LAYOUT_BF16X4, P2>) : fn(k_propagate_mixed<LAYOUT_BF16X4, P2>);
+    case LAYOUT_F32X4: return with_mixed_kernel_of<LAYOUT_F32X4, P2, true>(mod, fn);
+    case LAYOUT_BF16X4: return with_mixed_kernel_of<LAYOUT_BF16X4, P2, true>(mod, fn);
     case LAYOUT_F32_CELLS:
-        return mod ? fn(k_propagate_mixed_mod<LAYOUT_F32_CELLS, P2>) : fn(k_propagate_mixed<LAYOUT_F32_CELLS, P2>);
+        return pick ? with_mixed_kernel_of<LAYOUT_F32_CELLS, P2, true>(mod, fn)
+                    : with_mixed_kernel_of<LAYOUT_F32_CELLS, P2, false>(mod, fn);
     case LAYOUT_BF16_CELLS:
-        return mod ? fn(k_propagate_mixed_mod<LAYOUT_BF16_CELLS, P2>) : fn(k_propagate_mixed<LAYOUT_BF16_CELLS, P2>);
+        return pick ? with_mixed_kernel_of<LAYOUT_BF16_CELLS, P2, true>(mod, fn)
+                    : with_mixed_kernel_of<LAYOUT_BF16_CELLS, P2, false>(mod, fn);
     default: return (int)cudaErrorInvalidValue;
     }
 }
 
 template <typename Fn>
-int with_mixed_kernel(int layout, int mod, int p2, Fn&& fn) {
-    return p2 ? with_mixed_kernel_p2<true>(layout, mod, fn) : with_mixed_kernel_p2<false>(layout, mod, fn);
+int with_mixed_kernel(int layout, int mod, int p2, int pick, Fn&& fn) {
+    return p2 ? with_mixed_kernel_p2<true>(layout, mod, pick, fn) : with_mixed_kernel_p2<false>(layout, mod, pick, fn);
 }
 
 size_t mixed_smem(int mod, int block) { return (size_t)(kFieldWords + (mod ? kModSlots : 0)) * sizeof(float) * block; }
@@ -801,7 +809,7 @@ int launch_propagate_mixed(const PropArgs& a, int layout, int mod, int p2, int g
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const size_t shm = mixed_smem(mod, block);
     const int pct = mixed_carveout_pct(grid, shm);
-    return with_mixed_kernel(layout, mod, p2, [&](void (*k)(const PropArgs)) {
+    return with_mixed_kernel(layout, mod, p2, a.pickup, [&](void (*k)(const PropArgs)) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
         if (e != cudaSuccess) return (int)e;
         k<<<grid, block, shm, st>>>(a);
@@ -809,9 +817,9 @@ int launch_propagate_mixed(const PropArgs& a, int layout, int mod, int p2, int g
     });
 }
 
-int propagate_mixed_occupancy(int layout, int mod, int p2, int block, int* blocks_per_sm) {
+int propagate_mixed_occupancy(int layout, int mod, int p2, int pick, int block, int* blocks_per_sm) {
     const size_t shm = mixed_smem(mod, block);
-    return with_mixed_kernel(layout, mod, p2, [&](void (*k)(const PropArgs)) {
+    return with_mixed_kernel(layout, mod, p2, pick, [&](void (*k)(const PropArgs)) {
         // the query sees the driver's default carveout, not the one a previous launch chose
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, -1);
         if (e != cudaSuccess) return (int)e;
