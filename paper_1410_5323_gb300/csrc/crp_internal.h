@@ -126,7 +126,8 @@ int launch_arrival_map(const SimState& S, const Counters* C, int nside, double e
                        unsigned long long* map, int grid, void* stream);
 
 // Lenses (lens.cu).
-int launch_lens_apply(int n_pix, int n_maps, int group, const long long* rs, const int* rl, const int* col,
+// plain: every stored value is a normal number.
+int launch_lens_apply(int n_pix, int n_maps, int group, int plain, const long long* rs, const int* rl, const int* col,
                       const float* val, const double* x, double* y, int sms, void* stream);
 int launch_lens_bin(const SimState& S, const Counters* C, int nside, int n_mat, const double* edges, double e_min,
                     double* x, int grid, void* stream);

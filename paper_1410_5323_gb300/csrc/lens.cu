@@ -12,9 +12,9 @@
 // the stacked maps (n_mat x n_pix doubles per map) stay in L2.
 //   one map  : a group of G lanes per output row, each lane every G-th group of four
 //              entries of the row (rows padded to start on 16 bytes), the group reduces at
-//              the end (G from the mean merged row length);
-//   n_maps>1 : a warp per (row, 32 consecutive maps); lanes own maps, entries are read once
-//              per warp (broadcast), and every map sums its row in stored order.
+//              the end (G from the number of rows and the mean merged row length);
+//   n_maps>1 : as many rows per warp as their maps find lanes; lanes own maps, entries are read
+//              once per row (broadcast), and every map sums its row in stored order.
 // Compiled with --fmad=false; the fused multiply-adds are explicit.
 #include <cuda_runtime.h>
 
@@ -97,28 +97,93 @@ __global__ void __launch_bounds__(256) k_lens_apply_vec(int n_pix, const long lo
     }
 }
 
-__global__ void __launch_bounds__(256) k_lens_apply_maps(int n_pix, int n_maps, const long long* __restrict__ rs,
-                                                         const int* __restrict__ rl, const int* __restrict__ col,
-                                                         const float* __restrict__ val,
-                                                         const double* __restrict__ x, double* __restrict__ y) {
+// widen_f32 for normal values (a lens is PLAIN if all of its stored values are): four instructions.
+// (For one map, where the kernel waits on memory, it was no faster, and slower on a cold lens.)
+template <bool PLAIN>
+__device__ __forceinline__ double widen(float v) {
+    if constexpr (PLAIN) {
+        const int u = __float_as_int(v);
+        return __hiloint2double(((u >> 3) & (int)0x8FFFFFFF) + 0x38000000, (int)((unsigned)u << 29));
+    } else {
+        return widen_f32(v);
+    }
+}
+
+// Several maps: `width` lanes per row own one map each (b0 + lane), and a warp takes 32 / width rows.
+// The kernel is bound by one FP64 FMA per entry and map, and GB300 issues one FP64 warp instruction
+// per 64 cycles per sub-partition whatever its active lanes, so lanes without a map cost as much as
+// the others. A lane's sum is one dependent chain in stored order; while it takes up kPipe entries, the
+// maps' values of the next kPipe and the columns of those after them are on their way. (8, 12 and 16
+// were no faster, and with 32 maps 15 to 28 % slower for their registers.) Against one row per warp:
+// nside 64, 24 bins of 24, 10 maps 1551 -> 532 us (450 us of FP64 issue at 32 maps a warp); nside 32,
+// 16 maps 432 -> 218 us; nside 16, 12 bins of 20, 10 maps 62 -> 27 us, which is the longest row's chain.
+constexpr int kPipe = 4;
+
+template <bool PLAIN>
+__global__ void __launch_bounds__(64) k_lens_apply_maps(int n_pix, int n_maps, int b0, int width,
+                                                        const long long* __restrict__ rs, const int* __restrict__ rl,
+                                                        const int* __restrict__ col, const float* __restrict__ val,
+                                                        const double* __restrict__ x, double* __restrict__ y) {
     CRP_COUNT_RUN();
-    const int lane = threadIdx.x & 31;
-    const int chunks = (n_maps + 31) / 32;
-    const long long warps = (long long)gridDim.x * blockDim.x / 32;
-    for (long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32; w < (long long)n_pix * chunks;
-         w += warps) {
-        const long long p = w / chunks;
-        const int b = (int)(w % chunks) * 32 + lane;
-        const bool on = b < n_maps;
+    const int lane = threadIdx.x & 31, rows = 32 / width;
+    const int sub = lane / width;
+    if (sub >= rows) return;
+    const int b = b0 + lane - sub * width;
+    const double* xb = x + b;
+    const long long step = ((long long)gridDim.x * blockDim.x >> 5) * rows;
+    for (long long p = ((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5) * rows + sub; p < n_pix; p += step) {
+        const long long k0 = __ldg(rs + p);
+        const int len = __ldg(rl + p);
         double acc = 0.0;
-        const long long k0 = __ldg(rs + p), k1 = k0 + __ldg(rl + p);
-#pragma unroll 4
-        for (long long k = k0; k < k1; ++k) {
-            const double v = widen_f32(__ldg(val + k));
-            const int c = __ldg(col + k);
-            if (on) acc = __fma_rn(v, __ldg(x + (long long)c * n_maps + b), acc);
+        if (len > 0) {
+            // rows start on 16 bytes and are padded to multiples of four (column 0, never summed);
+            // vectors past the row's last repeat it
+            const int4* c4 = reinterpret_cast<const int4*>(col + k0);
+            const float4* v4 = reinterpret_cast<const float4*>(val + k0);
+            const int last = (len - 1) >> 2;
+            struct Ahead { double x[kPipe]; float v[kPipe]; } A, B;
+            int c[kPipe];
+            auto columns = [&](int k) {              // of the kPipe entries from k on
+#pragma unroll
+                for (int t = 0; t < kPipe; t += 4) {
+                    const int4 q = __ldg(c4 + min((k + t) >> 2, last));
+                    c[t] = q.x; c[t + 1] = q.y; c[t + 2] = q.z; c[t + 3] = q.w;
+                }
+            };
+            auto fetch = [&](Ahead& P, int k) {      // c holds the columns from k on
+#pragma unroll
+                for (int t = 0; t < kPipe; ++t) P.x[t] = __ldg(xb + (long long)c[t] * n_maps);
+#pragma unroll
+                for (int t = 0; t < kPipe; t += 4) {
+                    const float4 q = __ldg(v4 + min((k + t) >> 2, last));
+                    P.v[t] = q.x; P.v[t + 1] = q.y; P.v[t + 2] = q.z; P.v[t + 3] = q.w;
+                }
+                columns(k + kPipe);
+            };
+            auto take = [&](const Ahead& P) {
+#pragma unroll
+                for (int t = 0; t < kPipe; ++t) acc = __fma_rn(widen<PLAIN>(P.v[t]), P.x[t], acc);
+            };
+            columns(0);
+            fetch(A, 0);
+            int k = 0;
+            for (; k + 2 * kPipe <= len; k += 2 * kPipe) {
+                fetch(B, k + kPipe);
+                take(A);
+                fetch(A, k + 2 * kPipe);
+                take(B);
+            }
+            if (k + kPipe <= len) {
+                fetch(B, k + kPipe);
+                take(A);
+                A = B;
+                k += kPipe;
+            }
+#pragma unroll
+            for (int t = 0; t < kPipe; ++t)
+                if (k + t < len) acc = __fma_rn(widen<PLAIN>(A.v[t]), A.x[t], acc);
         }
-        if (on) y[p * n_maps + b] = acc;
+        y[p * n_maps + b] = acc;
     }
 }
 
@@ -147,11 +212,11 @@ __global__ void k_lens_bin(SimState S, const Counters* C, int nside, int n_mat, 
 
 }  // namespace
 
-int launch_lens_apply(int n_pix, int n_maps, int group, const long long* rs, const int* rl, const int* col,
-                      const float* val, const double* x, double* y, int sms, void* stream) {
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const int block = 256;
+template <bool PLAIN>
+void launch_apply(int n_pix, int n_maps, int group, const long long* rs, const int* rl, const int* col, const float* val,
+                  const double* x, double* y, int sms, cudaStream_t st) {
     if (n_maps == 1) {
+        const int block = 256;
         const long long threads = ((long long)n_pix * group + 31) / 32 * 32;
         long long blocks = (threads + block - 1) / block;
         const long long cap = (long long)sms * 8 * 16;
@@ -162,13 +227,25 @@ int launch_lens_apply(int n_pix, int n_maps, int group, const long long* rs, con
         case 16: k_lens_apply_vec<16><<<(int)blocks, block, 0, st>>>(n_pix, rs, rl, col, val, x, y); break;
         default: k_lens_apply_vec<32><<<(int)blocks, block, 0, st>>>(n_pix, rs, rl, col, val, x, y); break;
         }
-    } else {
-        const long long warps = (long long)n_pix * ((n_maps + 31) / 32);
-        long long blocks = (warps * 32 + block - 1) / block;
-        const long long cap = (long long)sms * 8 * 16;
-        if (blocks > cap) blocks = cap;
-        k_lens_apply_maps<<<(int)blocks, block, 0, st>>>(n_pix, n_maps, rs, rl, col, val, x, y);
+        return;
     }
+    // 32 maps at a time, then what is left of them
+    for (int b0 = 0; b0 < n_maps; b0 += 32) {
+        const int width = n_maps - b0 < 32 ? n_maps - b0 : 32;
+        const int rows = 32 / width;
+        const long long warps = ((long long)n_pix + rows - 1) / rows;
+        long long blocks = (warps + 1) / 2;          // two warps a block: few rows spread over all SMs
+        const long long cap = (long long)sms * 32 * 16;
+        if (blocks > cap) blocks = cap;
+        k_lens_apply_maps<PLAIN><<<(int)blocks, 64, 0, st>>>(n_pix, n_maps, b0, width, rs, rl, col, val, x, y);
+    }
+}
+
+int launch_lens_apply(int n_pix, int n_maps, int group, int plain, const long long* rs, const int* rl, const int* col,
+                      const float* val, const double* x, double* y, int sms, void* stream) {
+    const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    if (plain) launch_apply<true>(n_pix, n_maps, group, rs, rl, col, val, x, y, sms, st);
+    else launch_apply<false>(n_pix, n_maps, group, rs, rl, col, val, x, y, sms, st);
     return (int)cudaGetLastError();
 }
 

@@ -147,3 +147,29 @@ def test_full_size_lens_every_row(oracle_lib):
     assert np.all(np.abs(y - ref) <= _bound(n_pix, rp, col, val, x[:, :, None])[:, 0])
     x32 = np.random.default_rng(64).poisson(3.0, (24, n_pix, 32)).astype(np.float64)
     assert np.array_equal(_gpu(lens, x32), O.lens_apply(n_pix, rp, col, val, x32))
+
+
+@pytest.mark.parametrize("n_maps", [2, 3, 5, 10, 11, 16, 17, 31, 33, 42])
+def test_rows_packed_into_warps_bit_identical(oracle_lib, n_maps):
+    """Map counts that leave 0 to 16 rows per warp and lanes without a row, with rows of 0 to 40
+    entries around the lookahead, stored subnormals, zeros and infinities (the general widening),
+    and a number of rows that no warp size divides."""
+    import paper_1410_5323_gb300 as crp
+
+    rng = np.random.default_rng(n_maps)
+    n_pix, n_mat = 101, 2
+    counts = rng.integers(0, 21, (n_mat, n_pix))
+    counts[:, :9] = np.arange(9)
+    rp = np.zeros((n_mat, n_pix + 1), np.int64)
+    rp[0, 1:] = np.cumsum(counts[0])
+    rp[1, 0] = rp[0, -1]
+    rp[1, 1:] = rp[0, -1] + np.cumsum(counts[1])
+    nnz = int(rp[-1, -1])
+    col = rng.integers(0, n_pix, nnz).astype(np.int32)
+    val = (rng.standard_normal(nnz) * 10.0 ** rng.integers(-6, 6, nnz)).astype(np.float32)
+    x = rng.standard_normal((n_mat, n_pix, n_maps))
+    for special in (False, True):
+        if special:
+            val[rng.integers(0, nnz, 40)] = rng.choice(np.float32([0.0, -0.0, 1e-41, -3e-45, np.inf]), 40)
+        y = _gpu(crp.Lens(n_pix, rp, col, val), x)
+        assert np.array_equal(y, O.lens_apply(n_pix, rp, col, val, x), equal_nan=True)
