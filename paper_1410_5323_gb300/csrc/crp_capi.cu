@@ -1014,7 +1014,8 @@ int crp_source_sample(crp_sim* s, const crp_spectrum* sp, const double* x, const
         char* dst = (char*)*col_ptr(s->st, c.col) + f * kCols[c.col].size;
         CRP_CUDA(cudaMemcpyAsync(dst, c.src, (size_t)n * kCols[c.col].size, kind, st));
     }
-    int e = launch_source_sample(s->st, f, n, h.n_primaries, *sp, s->seed, grid_for(n, 128, 8192), st);
+    int e = launch_source_sample(s->st, f, n, h.n_primaries, *sp, s->seed,
+                                 grid_for(n, 128, 16 * std::max(1, s->sms)), st);
     if (e) return cuda_fail((cudaError_t)e, "source sampling kernel");
     const int block = 256;
     k_inject_init<<<grid_for(n, block, 4096), block, 0, st>>>(

@@ -197,14 +197,27 @@ __global__ void k_lens_bin(SimState S, const Counters* C, int nside, int n_mat, 
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         if (S.status[i] != CRP_STATUS_DONE_ || S.Z[i] <= 0 || !(S.E[i] > e_min)) continue;
-        const double R = S.E[i] / (double)S.Z[i];
-        if (!(edges[0] <= R && R < edges[n_mat])) continue;
+        // the bin by FP32 rigidity and edges (off by 2^-22 relative) unless R is that near one of them
+        const float R32 = sky::head_f32(S.E[i]) / (float)S.Z[i];
         int lo = 0, hi = n_mat;              // edges[lo] <= R < edges[hi]
         while (hi - lo > 1) {
             const int mid = (lo + hi) / 2;
-            if (edges[mid] <= R) lo = mid; else hi = mid;
+            if (sky::head_f32(edges[mid]) <= R32) lo = mid; else hi = mid;
         }
-        const long long p = sky::healpix_ring(nside, -S.ux[i], -S.uy[i], -S.uz[i]);
+        const float below = sky::head_f32(edges[lo]), above = sky::head_f32(edges[lo + 1]);
+        if (!(R32 > below * 1.000002f && R32 < above * 0.999998f)) {
+            if (lo == 0 && R32 < below * 0.999998f) continue;
+            if (lo == n_mat - 1 && R32 > above * 1.000002f) continue;
+            const double R = S.E[i] / (double)S.Z[i];
+            if (!(edges[0] <= R && R < edges[n_mat])) continue;
+            lo = 0;
+            hi = n_mat;
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) / 2;
+                if (edges[mid] <= R) lo = mid; else hi = mid;
+            }
+        }
+        const long long p = sky::healpix_pixel(nside, -S.ux[i], -S.uy[i], -S.uz[i]);
         if (p < 0 || p >= n_pix) continue;
         atomicAdd(x + (long long)lo * n_pix + p, 1.0);
     }

@@ -207,3 +207,44 @@ def test_full_size_sec4_workload_sampled_bit_identical_and_map(oracle_lib):
     u = -np.stack([gs["ux"][sel], gs["uy"][sel], gs["uz"][sel]], 1)
     ref = np.bincount(O.healpix_ring(w.arrival_nside, u), minlength=12 * w.arrival_nside ** 2)
     assert np.array_equal(amap, ref) and amap.sum() == sel.sum() > 0
+
+
+@pytest.mark.parametrize("species,alpha,rcut,lo,hi", [
+    (EQ1, 1.0, RCUT, 1e18, 1e21),                      # log-uniform
+    (EQ1, 0.3, RCUT, 1e18, 1e20),                      # rising
+    (EQ1, 4.5, 1e18, 1e17, 1e21),                      # steep: hi/lo far below FP32's resolution
+    (EQ1, 40.0, 1e19, 1e18, 1e21),                     # powers outside the FP32 range
+    (EQ1, 1.0000001, RCUT, 1e18, 1e21),                # nearly flat
+    ([(1, 1, 1.0)], 2.0, 3e17, 1e18, 1e21),            # most draws rejected
+    ([(4, 2, 0.0), (14, 7, 1e-30), (56, 26, 2e-30)], 2.0, 1e21, 1e19, 1.0001e19),
+    ([(a, (a + 1) // 2, 1.0 / a) for a in range(1, 9)], 2.3, 1e20, 1e18, 1e22),
+])
+def test_sampled_spectra_bit_identical(species, alpha, rcut, lo, hi):
+    """Draws tried in FP32 and kept in FP64 give the FP64 reading's particles for any spectrum."""
+    import paper_1410_5323_gb300 as crp
+
+    n = 20_011
+    sim, _ = _sim(n, seed=5)
+    sim.sample_sources(crp.Spectrum.of(species, alpha, rcut, lo, hi), np.zeros((n, 3)))
+    sim.sync(60.0, raise_on_error=False)
+    s = sim.state()
+    A, Z, E, u, _ = O.source_sample(O.spectrum(species, alpha, rcut, lo, hi), 5, 0, n)
+    assert np.array_equal(s["A"], A) and np.array_equal(s["Z"], Z)
+    assert np.array_equal(s["E"], E, equal_nan=True)
+    for c, k in (("ux", 0), ("uy", 1), ("uz", 2)):
+        assert np.array_equal(s[c], u[:, k])
+
+
+@pytest.mark.parametrize("nside", [3, 96, 512, 513])
+def test_healpix_pixels_on_both_sides_of_the_fp32_limit(oracle_lib, nside):
+    """300 000 random directions and the hard ones (borders, seams, poles, lengths far from one)."""
+    import paper_1410_5323_gb300 as crp
+    import torch
+
+    rng = np.random.default_rng(nside)
+    u = np.concatenate([rng.standard_normal((300_000, 3)), _hard_directions(nside, rng),
+                        rng.standard_normal((500, 3)) * 1e-25, rng.standard_normal((500, 3)) * 1e30,
+                        rng.standard_normal((200, 3)) * np.array([1e-12, 1e-12, 1.0]),
+                        rng.standard_normal((200, 3)) * np.array([1.0, 1e-45, 1.0])])
+    got = crp.healpix_ring(nside, torch.from_numpy(np.ascontiguousarray(u)).cuda()).cpu().numpy()
+    assert np.array_equal(got, O.healpix_ring(nside, u))
