@@ -3,11 +3,13 @@
 //
 // A forward pass with the adaptive Cash-Karp controller records the accepted step sizes
 // h_n and checkpoints y = (x, u) every K steps. The map y_{n+1} = y_n + h_n sum_i b_i k_i
-// is then differentiated exactly for fixed h_n: the states are recomputed from the
-// checkpoints (all segments in parallel into a stage-state buffer when the device has room,
-// else one segment at a time per particle), and the steps are reversed stage by stage with the
-// vector-Jacobian product of f(y) = (u, kappa u x B(x)), which also yields dL/dkappa and
-// scatters dL/dB into the grid gradient through the trilinear weights (FP64 atomics).
+// is then differentiated exactly for fixed h_n. When the device has room, the forward pass also
+// leaves the state at every step, and what the reverse sweep applies of each stage (a function of the
+// stage state alone) is formed for all steps in parallel in a buffer of stage records; else the
+// states are recomputed from the checkpoints, one segment at a time per particle. The steps are
+// reversed stage by stage with the vector-Jacobian product of f(y) = (u, kappa u x B(x)), which also
+// yields dL/dkappa and scatters dL/dB into the grid gradient through the trilinear weights (FP64
+// atomics).
 // Compiled with --fmad=false; per-particle arithmetic follows the oracle's order.
 #include <cuda_runtime.h>
 
@@ -16,6 +18,7 @@
 #include "crp_fp64.cuh"
 #include "crp_internal.h"
 #include "crp_math.cuh"
+#include "crp_team.cuh"
 
 // Runs of this file's kernels (diagnostics: each launch adds one, from its first thread).
 namespace {
@@ -100,7 +103,17 @@ __device__ __forceinline__ void lookup_jac(const FieldDev& F, double x, double y
     axis<P2>(x, F.oix, F.inv_spacing, F.nx, F.pow2, ix[0], ix[1], wx[0], wx[1]);
     axis<P2>(y, F.oiy, F.inv_spacing, F.ny, F.pow2, iy[0], iy[1], wy[0], wy[1]);
     axis<P2>(z, F.oiz, F.inv_spacing, F.nz, F.pow2, iz[0], iz[1], wz[0], wz[1]);
-    const double dd[2] = {-F.inv_spacing, F.inv_spacing};
+    // the derivative products without their sign ((-1/spacing) w w' is exactly -((1/spacing) w w'))
+    double dx[2][2], dy[2][2], dz[2][2];
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+        const double sx = F.inv_spacing * wy[b], sy = wx[b] * F.inv_spacing;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            dx[b][c] = sx * wz[c];
+            dy[b][c] = sy * wz[c];
+        }
+    }
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
         o.B[q] = 0.0;
@@ -111,12 +124,13 @@ __device__ __forceinline__ void lookup_jac(const FieldDev& F, double x, double y
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int b = 0; b < 2; ++b)
+        for (int b = 0; b < 2; ++b) {
+            const double wab = wx[a] * wy[b];
+            dz[a][b] = wab * F.inv_spacing;
 #pragma unroll
             for (int c = 0; c < 2; ++c, ++c8) {
-                const double wab = wx[a] * wy[b];
                 const double wt = wab * wz[c];
-                const double dw[3] = {(dd[a] * wy[b]) * wz[c], (wx[a] * dd[b]) * wz[c], wab * dd[c]};
+                const double dw[3] = {a ? dx[b][c] : -dx[b][c], b ? dy[a][c] : -dy[a][c], c ? dz[a][b] : -dz[a][b]};
                 o.w[c8] = wt;
                 o.node[c8] = (ix[a] * F.ny + iy[b]) * F.nz + iz[c];
                 const V3 g = corner<L>(F, o.node[c8]);
@@ -128,6 +142,7 @@ __device__ __forceinline__ void lookup_jac(const FieldDev& F, double x, double y
                     for (int d = 0; d < 3; ++d) o.J[q][d] = __fma_rn(dw[d], G[q], o.J[q][d]);
                 }
             }
+        }
 }
 
 // Vector-Jacobian product of f(Y) = (u, kappa u x B(x)) with cotangent kb = (abar, bbar), from
@@ -269,25 +284,25 @@ __device__ __forceinline__ Y6 deriv_from(double kappa, const Y6& y, const Look& 
     return k;
 }
 
-// Stage records of the segments [sg0, sg0 + n_seg): thread (particle i, segment sg)
-// recomputes its segment from the checkpoint. Each step evaluates f at its six stage states
-// with the forward stage sums (as ck_attempt) and advances y by the 5th-order update, so the
-// states are the frozen forward's, bit for bit.
+// Stage records of the steps [m0, m0 + n_m): thread (particle i, step m) starts from the state that the
+// forward pass left at the step's start, and evaluates f at the six stage states with the forward
+// stage sums (as ck_attempt), so the states are the frozen forward's, bit for bit. With only the
+// checkpoints a thread went through a whole segment, 300 chains of 40 steps had 300 threads, and the
+// backward pass took 2.43 ms instead of 0.56. FP64 issue bounds it: 4096 chains of 2000 steps 22.5 ->
+// 14.8 ms in all, 16 products fewer in each of the six lookups and no recomputed step.
 template <int L, bool P2>
 __global__ void k_adj_records(FieldDev F, const double* __restrict__ kap, const double* __restrict__ h,
-                              const double* __restrict__ ck, double* __restrict__ rec_d,
-                              int32_t* __restrict__ rec_n, int n_steps, int K, int sg0, int n_seg,
-                              long long n) {
+                              const double* __restrict__ states, double* __restrict__ rec_d,
+                              int32_t* __restrict__ rec_n, int m0, int n_m, long long n) {
     CRP_COUNT_RUN();
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (t >= n * n_seg) return;
+    if (t >= n * n_m) return;
     const long long i = t % n;
-    const int sg = sg0 + (int)(t / n);
+    const int m = m0 + (int)(t / n);
     const double kappa = kap[i];
-    const int m0 = sg * K, m1 = min(m0 + K, n_steps);
     Y6 y;
-    load6(ck + (long long)sg * 6 * n, n, i, y);
-    for (int m = m0; m < m1; ++m) {
+    load6(states + (long long)m * 6 * n, n, i, y);
+    {
         const double h_ = h[(long long)m * n + i];
         Look o;
         Y6 t_;
@@ -324,18 +339,12 @@ __global__ void k_adj_records(FieldDev F, const double* __restrict__ kap, const 
         ADJ_STAGE(t_, R6);
         lookup_jac<L, P2>(F, t_.x, t_.y, t_.z, o);
         put_rec(rec_d, rec_n, n, i, m, 5, t_, o);
-        const Y6 k6 = deriv_from(kappa, t_, o);
-#define RB(c) __fma_rn(B6, k6.c, __fma_rn(B4, k4.c, __fma_rn(B3, k3.c, B1 * k1.c)))
-        Y6 y5;
-        ADJ_STAGE(y5, RB);
-        y = y5;
 #undef ADJ_STAGE
 #undef R2
 #undef R3
 #undef R4
 #undef R5
 #undef R6
-#undef RB
     }
 }
 
@@ -403,70 +412,17 @@ __global__ void k_adj_p0bar(const double* __restrict__ y0, const double* __restr
 // the corner weights, B_c and the c-th Lorentz component. Values of the whole particle (error
 // sums, accept decision, step size, kappa_bar) are formed by the same operations in all three
 // lanes. Every value is the one the one-lane form computes, so the results are the same bits.
-constexpr int kTeams = 10;
+constexpr int kTeams = kTeamsPerWarp;
 
 struct Team {
     unsigned mask;   // the team's lanes
     int l0, c;       // its first lane, this lane's component
-    double oi;       // origin / spacing along axis c (rounded once), grid size along it
-    int nn;
     __device__ __forceinline__ double get(double v, int k) const { return __shfl_sync(mask, v, l0 + k); }
-    __device__ __forceinline__ long long get(long long v, int k) const { return __shfl_sync(mask, v, l0 + k); }
     __device__ __forceinline__ int nx1() const { return c == 2 ? 0 : c + 1; }
     __device__ __forceinline__ int nx2() const { return c == 0 ? 2 : c - 1; }
 };
 
-// B_c at the team's stage position (lane c holds its coordinate xc): the periodic trilinear
-// lookup of field_b, with the axes, the corner weights and the corner loads split over the
-// team. FP64 node copy: component c of node k at ((const double*)data)[4k + c].
-template <bool P2>
-__device__ __forceinline__ double field_team(const FieldDev& F, const Team& T, double xc) {
-    long long i0, i1;
-    const double oi = T.oi;
-    const int nn = T.nn;
-    double w0, w1;
-    axis<P2>(xc, oi, F.inv_spacing, nn, F.pow2, i0, i1, w0, w1);
-    const long long ix0 = T.get(i0, 0), ix1 = T.get(i1, 0), iy0 = T.get(i0, 1), iy1 = T.get(i1, 1);
-    const long long iz0 = T.get(i0, 2), iz1 = T.get(i1, 2);
-    const double wx0 = T.get(w0, 0), wx1 = T.get(w1, 0), wy0 = T.get(w0, 1), wy1 = T.get(w1, 1);
-    const double wz0 = T.get(w0, 2), wz1 = T.get(w1, 2);
-    // lane 0 forms w00, w01 and t0..t3, lane 1 w10, w11 and t4..t7 (lane 2 repeats lane 1)
-    const double wxa = T.c == 0 ? wx0 : wx1;
-    const double wA = wxa * wy0, wB = wxa * wy1;
-    const double tA0 = wA * wz0, tA1 = wA * wz1, tB0 = wB * wz0, tB1 = wB * wz1;
-    const double t0 = T.get(tA0, 0), t1 = T.get(tA1, 0), t2 = T.get(tB0, 0), t3 = T.get(tB1, 0);
-    const double t4 = T.get(tA0, 1), t5 = T.get(tA1, 1), t6 = T.get(tB0, 1), t7 = T.get(tB1, 1);
-    const long long ny = F.ny, nz = F.nz;
-    const long long r00 = (ix0 * ny + iy0) * nz, r01 = (ix0 * ny + iy1) * nz;
-    const long long r10 = (ix1 * ny + iy0) * nz, r11 = (ix1 * ny + iy1) * nz;
-    const double* G = reinterpret_cast<const double*>(F.data) + T.c;
-    const double g0 = __ldg(G + 4 * (r00 + iz0)), g1 = __ldg(G + 4 * (r00 + iz1));
-    const double g2 = __ldg(G + 4 * (r01 + iz0)), g3 = __ldg(G + 4 * (r01 + iz1));
-    const double g4 = __ldg(G + 4 * (r10 + iz0)), g5 = __ldg(G + 4 * (r10 + iz1));
-    const double g6 = __ldg(G + 4 * (r11 + iz0)), g7 = __ldg(G + 4 * (r11 + iz1));
-    double B = __fma_rn(t0, g0, 0.0);
-    B = __fma_rn(t1, g1, B);
-    B = __fma_rn(t2, g2, B);
-    B = __fma_rn(t3, g3, B);
-    B = __fma_rn(t4, g4, B);
-    B = __fma_rn(t5, g5, B);
-    B = __fma_rn(t6, g6, B);
-    B = __fma_rn(t7, g7, B);
-    return B;
-}
-
-// Component c of f(Y) = (u, kappa u x B(x)): (ku_c = kappa fma(u_{c+1}, B_{c+2}, -(u_{c+2} B_{c+1}))).
-template <bool P2>
-__device__ __forceinline__ void deriv_team(const FieldDev& F, const Team& T, double kappa, double yx,
-                                           double yu, double& kx, double& ku) {
-    const double B = field_team<P2>(F, T, yx);
-    const double u1 = T.get(yu, T.nx1()), u2 = T.get(yu, T.nx2());
-    const double B1 = T.get(B, T.nx1()), B2 = T.get(B, T.nx2());
-    kx = yu;
-    ku = kappa * __fma_rn(u1, B2, -(u2 * B1));
-}
-
-__device__ __forceinline__ Team make_team(long long n, long long& i, bool& active, const FieldDev* F = nullptr) {
+__device__ __forceinline__ Team make_team(long long n, long long& i, bool& active) {
     const int lane = threadIdx.x & 31;
     const int team = lane / 3;
     const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
@@ -476,100 +432,93 @@ __device__ __forceinline__ Team make_team(long long n, long long& i, bool& activ
     T.l0 = 3 * team;
     T.c = lane - T.l0;
     T.mask = 7u << T.l0;
-    T.oi = 0.0;
-    T.nn = 1;
-    if (F) {
-        T.oi = T.c == 0 ? F->oix : (T.c == 1 ? F->oiy : F->oiz);
-        T.nn = T.c == 0 ? F->nx : (T.c == 1 ? F->ny : F->nz);
-    }
     return T;
 }
 
-// Forward with the propagation module's controller only, in team form; records h_n and the
-// checkpoints of every K-th step (the oracle's frozen forward, value for value).
+// Forward with the propagation module's controller only, in team form (the lookups, attempts and error
+// sums of crp_team.cuh; all lanes of a warp together); records h_n, the checkpoints of every K-th step
+// and, if `states` is not NULL, the state at the start of every step (the oracle's frozen forward,
+// value for value). Chains are dealt out evenly, `per_warp` to a warp: warps that share a
+// sub-partition share its FP64 unit.
 template <bool P2>
-__global__ void k_adj_record_team(FieldDev F, const double* __restrict__ y0, const double* __restrict__ kap,
-                                  double tol, double hmin, double hmax, int n_steps, int K,
-                                  double* __restrict__ h_out, double* __restrict__ ck,
-                                  double* __restrict__ xT, double* __restrict__ uT, long long n) {
+__global__ void __launch_bounds__(128) k_adj_record_team(FieldDev F, const double* __restrict__ y0,
+                                                         const double* __restrict__ kap, double tol, double hmin,
+                                                         double hmax, int n_steps, int K, int per_warp,
+                                                         double* __restrict__ h_out, double* __restrict__ ck,
+                                                         double* __restrict__ states, double* __restrict__ xT,
+                                                         double* __restrict__ uT, long long n) {
     CRP_COUNT_RUN();
-    long long i;
-    bool active;
-    const Team T = make_team(n, i, active, &F);
-    if (!active) return;
+    const team::Lane T = team::lane_of_team();
     const int c = T.c;
-    double yx = y0[(long long)c * n + i], yu = y0[(long long)(3 + c) * n + i];
-    const double kappa = kap[i];
+    const int t = (threadIdx.x & 31) / 3;
+    const long long i = ((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5) * per_warp + t;
+    const bool active = t < per_warp && i < n;
+    const double* data = static_cast<const double*>(F.data) + (active ? c : 0);
+    const team::Axis V = active ? team::vector_axis(F, c) : team::parked_axis();
+    double yx = 0.0, yu = 0.0, kappa = 0.0;
+    if (active) {
+        yx = y0[(long long)c * n + i];
+        yu = y0[(long long)(3 + c) * n + i];
+        kappa = kap[i];
+    }
     const double tol2 = tol * tol;
     const float lg_tol = ctrl_log2(tol);
     // one attempt per iteration: teams that retry a step and teams that start one run the
     // attempt together (a rejection in one team does not make the warp repeat it for the rest)
     double hprop = __longlong_as_double(0x7ff0000000000000LL);
-    double h = 0.0, h_prop = 0.0, k1x = 0.0, k1u = 0.0;
-    int m = 0, rejected = 0;
-    bool new_step = true;
-    while (m < n_steps) {
+    double h = 0.0, h_prop = 0.0, k1u = 0.0;
+    int m = active ? 0 : n_steps, rejected = 0, to_ck = 0;
+    bool new_step = active;
+    auto deriv = [&](double x, double u) { return team::force_c(T, kappa, u, team::field_c<P2>(data, V, T, x)); };
+    while (__any_sync(kFull, m < n_steps)) {
         if (new_step) {
-            if (m % K == 0) {
+            if (to_ck == 0) {
                 double* q = ck + (long long)(m / K) * 6 * n;
+                q[(long long)c * n + i] = yx;
+                q[(long long)(3 + c) * n + i] = yu;
+                to_ck = K;
+            }
+            to_ck -= 1;
+            if (states) {
+                double* q = states + (long long)m * 6 * n;
                 q[(long long)c * n + i] = yx;
                 q[(long long)(3 + c) * n + i] = yu;
             }
             h_prop = clampd(hprop, hmin, hmax);
             h = h_prop;
-            deriv_team<P2>(F, T, kappa, yx, yu, k1x, k1u);
             rejected = 0;
+        }
+        __syncwarp();
+        if (__any_sync(kFull, new_step)) {
+            const double k1n = deriv(yx, yu);
+            if (new_step) k1u = k1n;
             new_step = false;
         }
-        double tx, tu, k2x, k2u, k3x, k3u, k4x, k4u, k5x, k5u, k6x, k6u;
-        tx = __fma_rn(h, A21 * k1x, yx); tu = __fma_rn(h, A21 * k1u, yu);
-        deriv_team<P2>(F, T, kappa, tx, tu, k2x, k2u);
-#define T3(k) __fma_rn(A32, k2##k, A31 * k1##k)
-        tx = __fma_rn(h, T3(x), yx); tu = __fma_rn(h, T3(u), yu);
-        deriv_team<P2>(F, T, kappa, tx, tu, k3x, k3u);
-#define T4(k) __fma_rn(A43, k3##k, __fma_rn(A42, k2##k, A41 * k1##k))
-        tx = __fma_rn(h, T4(x), yx); tu = __fma_rn(h, T4(u), yu);
-        deriv_team<P2>(F, T, kappa, tx, tu, k4x, k4u);
-#define T5(k) __fma_rn(A54, k4##k, __fma_rn(A53, k3##k, __fma_rn(A52, k2##k, A51 * k1##k)))
-        tx = __fma_rn(h, T5(x), yx); tu = __fma_rn(h, T5(u), yu);
-        deriv_team<P2>(F, T, kappa, tx, tu, k5x, k5u);
-#define T6(k) __fma_rn(A65, k5##k, __fma_rn(A64, k4##k, __fma_rn(A63, k3##k, __fma_rn(A62, k2##k, A61 * k1##k))))
-        tx = __fma_rn(h, T6(x), yx); tu = __fma_rn(h, T6(u), yu);
-        deriv_team<P2>(F, T, kappa, tx, tu, k6x, k6u);
-#define TB(k) __fma_rn(B6, k6##k, __fma_rn(B4, k4##k, __fma_rn(B3, k3##k, B1 * k1##k)))
-#define TE(k) (h * __fma_rn(E6, k6##k, __fma_rn(E5, k5##k, __fma_rn(E4, k4##k, __fma_rn(E3, k3##k, E1 * k1##k)))))
-        const double y5x = __fma_rn(h, TB(x), yx), y5u = __fma_rn(h, TB(u), yu);
-        const double ex = TE(x), eu = TE(u);
-#undef T3
-#undef T4
-#undef T5
-#undef T6
-#undef TB
-#undef TE
-        // squared norms ((e0^2 + e1^2) + e2^2) with fused products, as error_sums
-        const double ex0 = T.get(ex, 0), ex1 = T.get(ex, 1), ex2 = T.get(ex, 2);
-        const double eu0 = T.get(eu, 0), eu1 = T.get(eu, 1), eu2 = T.get(eu, 2);
-        const double sx = __fma_rn(ex2, ex2, __fma_rn(ex1, ex1, ex0 * ex0));
-        const double su = __fma_rn(eu2, eu2, __fma_rn(eu1, eu1, eu0 * eu0));
-        if (!(error_accept(sx, su, h, tol, tol2) || le_pos(h, hmin))) {
-            const float shrink = ctrl_factor(ctrl_log2r(sx, su, h, lg_tol), -0.25f, 0.1f, 1.0f);
-            h = max_pos(h * widen_normal(shrink), hmin);
-            rejected = 1;
-            continue;
+        double y5x, y5u, ex, eu, sx, su;
+        team::attempt_c(h, yx, yu, k1u, deriv, y5x, y5u, ex, eu);
+        team::error_sums_t(T, ex, eu, sx, su);
+        if (m < n_steps) {
+            const bool accept = error_accept(sx, su, h, tol, tol2) || le_pos(h, hmin);
+            const double hnew = h * widen_normal(step_factor(accept, sx, su, h, lg_tol));
+            if (accept) {
+                yx = y5x;
+                yu = y5u;
+                if (c == 0) h_out[(long long)m * n + i] = h;
+                double hnext = hnew;
+                if (!rejected && lt_pos(h, h_prop)) hnext = max_pos(hnext, h_prop);
+                hprop = clampd(hnext, hmin, hmax);
+                ++m;
+                new_step = m < n_steps;
+            } else {
+                h = max_pos(hnew, hmin);
+                rejected = 1;
+            }
         }
-        yx = y5x;
-        yu = y5u;
-        if (c == 0) h_out[(long long)m * n + i] = h;
-        const float grow = (is_zero(h) || (is_zero(sx) && is_zero(su)))
-                               ? 5.0f : ctrl_factor(ctrl_log2r(sx, su, h, lg_tol), -0.2f, 0.2f, 5.0f);
-        double hnext = h * widen_normal(grow);
-        if (!rejected && lt_pos(h, h_prop)) hnext = max_pos(hnext, h_prop);
-        hprop = clampd(hnext, hmin, hmax);
-        ++m;
-        new_step = true;
     }
-    xT[3 * i + c] = yx;
-    uT[3 * i + c] = yu;
+    if (active) {
+        xT[3 * i + c] = yx;
+        uT[3 * i + c] = yu;
+    }
 }
 
 // Reverse sweep over the stage records in team form: lane c owns component c of the cotangents.
@@ -690,6 +639,16 @@ __global__ void k_adj_reverse_team(const double* __restrict__ kap, const double*
     if (c == 0) kappa_bar_out[i] = kappa_bar;
 }
 
+long long device_sms_or_1() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
+        cudaGetLastError();
+        sms = 1;
+    }
+    return sms;
+}
+
 int team_blocks(long long n) { return (int)((n + kTeams - 1) / kTeams); }   // one warp per block
 
 int blocks(long long n) { return (int)((n + 127) / 128); }
@@ -709,11 +668,20 @@ int adj_init(const double* x0, const double* p0, const int32_t* Z, double* y0, d
 }
 
 int adj_record(const FieldDev& F, const double* y0, const double* kappa, double tol, double hmin,
-               double hmax, int n_steps, int K, double* h, double* ck, double* xT, double* uT,
+               double hmax, int n_steps, int K, double* h, double* ck, double* states, double* xT, double* uT,
                long long n, void* stream) {
     auto k = F.pow2 ? k_adj_record_team<true> : k_adj_record_team<false>;
-    k<<<team_blocks(n), 32, 0, (cudaStream_t)stream>>>(F, y0, kappa, tol, hmin, hmax, n_steps, K, h, ck,
-                                                        xT, uT, n);
+    const long long sms = device_sms_or_1();
+    const int per_warp = (int)std::max(1ll, std::min<long long>(kTeams, (n + 4 * sms - 1) / (4 * sms)));
+    const long long warps = (n + per_warp - 1) / per_warp;
+    // up to one block per SM: shared memory that a second one finds no room for spreads them
+    const int shm = warps <= 4 * sms ? 116 * 1024 : 0;
+    if (shm) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, shm);
+        if (e != cudaSuccess) return (int)e;
+    }
+    k<<<(unsigned)((warps + 3) / 4), 128, shm, (cudaStream_t)stream>>>(F, y0, kappa, tol, hmin, hmax, n_steps, K, per_warp,
+                                                                      h, ck, states, xT, uT, n);
     return (int)cudaGetLastError();
 }
 
@@ -728,30 +696,23 @@ int adj_replay(const FieldDev& F, const double* y0, const double* kappa, const d
     return (int)cudaGetLastError();
 }
 
-int adj_backward(const FieldDev& F, const double* kappa, const double* h, const double* ck,
+int adj_backward(const FieldDev& F, const double* kappa, const double* h, const double* ck, const double* states,
                  double* seg, double* stages, int n_steps, int K, const double* uT_bar, double* grid_bar,
                  double* y0_bar, double* kappa_bar, long long n, void* stream, void* aux_stream,
                  void* const* events, int n_events) {
     if (stages) {
-        // Stage records in chunks of checkpoint segments, last chunk first, on the auxiliary
-        // stream; the reverse sweep takes each chunk once its event has fired. The records
-        // kernel (FP64-throughput-bound, many threads) then runs beside the reverse sweep
-        // (one warp per ten chains, latency-bound). Without an auxiliary stream: one chunk.
-        // A chunk of C segments is n * C threads; C is the smallest that still gives every SM
-        // about one 128-thread block (fewer blocks leave SMs idle for the chunk's whole run).
+        // Stage records in chunks of steps, last chunk first, on the auxiliary stream; the reverse
+        // sweep takes each chunk once its event has fired. The records kernel
+        // (FP64-throughput-bound, many threads) then runs beside the reverse sweep (one warp per ten
+        // chains, latency-bound). Without an auxiliary stream: one chunk. A chunk gives every SM at
+        // least two 128-thread blocks; the first one, which the sweep waits for, a third of the others.
         const cudaStream_t st = (cudaStream_t)stream, aux = (cudaStream_t)aux_stream;
-        const int S = (n_steps + K - 1) / K;
-        int dev = 0, sms = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
-            cudaGetLastError();
-            sms = 1;
-        }
-        const long long c_min = std::max(1ll, (long long)((0.8 * sms * 128.0 + (double)n - 1.0) / (double)n));
-        int J = (aux && n_events >= 2) ? (int)std::min<long long>(n_events - 1, S / c_min) : 1;
+        const long long sms = device_sms_or_1();
+        const int c_min = (int)std::min<long long>(n_steps, (sms * 256 + n - 1) / n);
+        int J = (aux && n_events >= 2) ? std::min(n_events - 1, n_steps / c_min) : 1;
         J = std::max(1, J);
-        const int C = (S + J - 1) / J;
-        J = (S + C - 1) / C;
+        const int first = J > 1 ? std::max(c_min, n_steps / (3 * J)) : n_steps;
+        const int C = J > 1 ? std::max(c_min, (n_steps - first + J - 2) / (J - 1)) : n_steps;
         double* rec_d = stages;
         int32_t* rec_n = reinterpret_cast<int32_t*>(stages + (size_t)n_steps * 6 * kRecD * (size_t)n);
         const cudaStream_t rs = J > 1 ? aux : st;
@@ -761,23 +722,33 @@ int adj_backward(const FieldDev& F, const double* kappa, const double* h, const 
             if (e == cudaSuccess) e = cudaStreamWaitEvent(aux, (cudaEvent_t)events[0], 0);
             if (e != cudaSuccess) return (int)e;
         }
+        auto chunk = [&](int j, int& lo, int& hi) {      // the last one takes what is left
+            hi = j == 0 ? n_steps : n_steps - first - (j - 1) * C;
+            lo = j == J - 1 ? 0 : n_steps - first - j * C;
+            hi = std::max(hi, 0);
+            lo = std::max(lo, 0);
+        };
         for (int j = 0; j < J; ++j) {
-            const int hi = S - j * C, lo = std::max(0, hi - C);
-            auto k = F.pow2 ? k_adj_records<LAYOUT_F64X4, true> : k_adj_records<LAYOUT_F64X4, false>;
-            k<<<blocks(n * (hi - lo)), 128, 0, rs>>>(F, kappa, h, ck, rec_d, rec_n, n_steps, K, lo, hi - lo, n);
-            e = cudaGetLastError();
+            int lo, hi;
+            chunk(j, lo, hi);
+            if (hi > lo) {
+                auto k = F.pow2 ? k_adj_records<LAYOUT_F64X4, true> : k_adj_records<LAYOUT_F64X4, false>;
+                k<<<blocks(n * (hi - lo)), 128, 0, rs>>>(F, kappa, h, states, rec_d, rec_n, lo, hi - lo, n);
+                e = cudaGetLastError();
+            }
             if (e == cudaSuccess && J > 1) e = cudaEventRecord((cudaEvent_t)events[1 + j], aux);
             if (e != cudaSuccess) return (int)e;
         }
         for (int j = 0; j < J; ++j) {
-            const int hi = S - j * C, lo = std::max(0, hi - C);
+            int lo, hi;
+            chunk(j, lo, hi);
+            if (hi <= lo) continue;
             if (J > 1) {
                 e = cudaStreamWaitEvent(st, (cudaEvent_t)events[1 + j], 0);
                 if (e != cudaSuccess) return (int)e;
             }
-            k_adj_reverse_team<<<team_blocks(n), 32, 0, st>>>(
-                kappa, h, rec_d, rec_n, std::min(hi * K, n_steps), lo * K, j == 0 ? 1 : 0, uT_bar,
-                grid_bar, y0_bar, kappa_bar, n);
+            k_adj_reverse_team<<<team_blocks(n), 32, 0, st>>>(kappa, h, rec_d, rec_n, hi, lo, j == 0 ? 1 : 0, uT_bar,
+                                                              grid_bar, y0_bar, kappa_bar, n);
             e = cudaGetLastError();
             if (e != cudaSuccess) return (int)e;
         }

@@ -1903,6 +1903,7 @@ struct crp_adjoint {
     double *y0 = nullptr, *kappa = nullptr, *E = nullptr, *h = nullptr, *ck = nullptr;
     double *seg = nullptr, *y0_bar = nullptr, *kappa_bar = nullptr, *y0_tmp = nullptr;
     double *kappa_tmp = nullptr, *E_tmp = nullptr;
+    double* states = nullptr;            // state at the start of every step, kept with the stage records
     double* stages = nullptr;            // stage records of every step (kAdjRecordBytes each), if room
     int32_t* Z = nullptr;
     bool recorded = false;
@@ -1917,7 +1918,7 @@ namespace {
 
 void adj_free(crp_adjoint* a) {
     double* ds[] = {a->y0, a->kappa, a->E, a->h, a->ck, a->seg, a->y0_bar, a->kappa_bar, a->y0_tmp,
-                    a->kappa_tmp, a->E_tmp, a->stages};
+                    a->kappa_tmp, a->E_tmp, a->stages, a->states};
     for (double* p : ds)
         if (p) cudaFree(p);
     if (a->Z) cudaFree(a->Z);
@@ -1960,9 +1961,15 @@ int crp_adjoint_create(const crp_field* field, int64_t n, int32_t n_steps, int32
     // then formed in parallel and the serial reverse sweep only applies them
     size_t free_b = 0, total_b = 0;
     const size_t st_bytes = kAdjRecordBytes * (size_t)n_steps * (size_t)n;
+    const size_t y_bytes = 6 * sizeof(double) * (size_t)n_steps * (size_t)n;
     const long long nodes = (long long)F.nx * F.ny * F.nz;
-    if (nodes < (1ll << 31) && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && st_bytes <= free_b / 2) {
+    if (nodes < (1ll << 31) && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && st_bytes + y_bytes <= free_b / 2) {
         if (dev_malloc(&a->stages, st_bytes) != cudaSuccess) {
+            a->stages = nullptr;
+            cudaGetLastError();
+        } else if (dev_malloc(&a->states, y_bytes) != cudaSuccess) {
+            a->states = nullptr;
+            cudaFree(a->stages);
             a->stages = nullptr;
             cudaGetLastError();
         }
@@ -2002,7 +2009,7 @@ int crp_adjoint_forward(crp_adjoint* a, const double* x0, const double* p0, cons
     CRP_CUDA(cudaMemcpyAsync(a->Z, Z, sizeof(int32_t) * a->n, cudaMemcpyDeviceToDevice, st));
     int e = adj_init(x0, p0, a->Z, a->y0, a->kappa, a->E, a->n, st);
     if (e) return cuda_fail((cudaError_t)e, "adjoint init");
-    e = adj_record(F, a->y0, a->kappa, tol, hmin, hmax, a->n_steps, a->K, a->h, a->ck, xT, uT, a->n, st);
+    e = adj_record(F, a->y0, a->kappa, tol, hmin, hmax, a->n_steps, a->K, a->h, a->ck, a->states, xT, uT, a->n, st);
     if (e) return cuda_fail((cudaError_t)e, "adjoint forward");
     a->recorded = true;
     return CRP_OK;
@@ -2044,7 +2051,7 @@ int crp_adjoint_backward(crp_adjoint* a, const double* uT_bar, double* grid_bar,
     int rc = field_fp64_desc(a->field, F);
     if (rc) return rc;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    int e = adj_backward(F, a->kappa, a->h, a->ck, a->seg, a->stages, a->n_steps, a->K, uT_bar, grid_bar,
+    int e = adj_backward(F, a->kappa, a->h, a->ck, a->states, a->seg, a->stages, a->n_steps, a->K, uT_bar, grid_bar,
                          a->y0_bar, a->kappa_bar, a->n, st, a->aux, reinterpret_cast<void* const*>(a->ev),
                          a->n_ev);
     if (e) return cuda_fail((cudaError_t)e, "adjoint backward");

@@ -160,21 +160,22 @@ unsigned long long kernel_runs_sources();
 unsigned long long kernel_runs_lens();
 
 // Adjoint launchers (adjoint.cu). Arrays are component-major [component][n] for y,
-// [step][n] for h, [checkpoint][6][n] for checkpoints. `stages`, when not NULL, holds the
+// [step][n] for h, [checkpoint][6][n] for checkpoints,
+// [step][6][n] for `states` (the state at every step's start, kept with the stage records). `stages`, when not NULL, holds the
 // stage records of every step: per step and particle kAdjRecordBytes (6 stages x (23 FP64:
 // direction, field, Jacobian, corner weights + 8 int32 corner nodes)), doubles first.
 constexpr size_t kAdjRecordBytes = 6 * (23 * sizeof(double) + 8 * sizeof(int32_t));
 int adj_init(const double* x0, const double* p0, const int32_t* Z, double* y0, double* kappa,
              double* E, long long n, void* stream);
 int adj_record(const FieldDev& F, const double* y0, const double* kappa, double tol, double hmin,
-               double hmax, int n_steps, int K, double* h, double* ck, double* xT, double* uT,
+               double hmax, int n_steps, int K, double* h, double* ck, double* states, double* xT, double* uT,
                long long n, void* stream);
 int adj_replay(const FieldDev& F, const double* y0, const double* kappa, const double* h, int n_steps,
                double* xT, double* uT, unsigned long long* cell_hash, long long n, void* stream);
 // With `stages`, the records are formed in up to n_events - 1 chunks on `aux_stream` (events[0]
 // orders it after `stream`, events[1 + j] hands chunk j to the reverse sweep on `stream`);
 // aux_stream NULL: one chunk on `stream`.
-int adj_backward(const FieldDev& F, const double* kappa, const double* h, const double* ck,
+int adj_backward(const FieldDev& F, const double* kappa, const double* h, const double* ck, const double* states,
                  double* seg, double* stages, int n_steps, int K, const double* uT_bar, double* grid_bar,
                  double* y0_bar, double* kappa_bar, long long n, void* stream, void* aux_stream,
                  void* const* events, int n_events);

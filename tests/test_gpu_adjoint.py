@@ -312,3 +312,34 @@ def test_team_sweeps_with_partial_teams_match_the_oracle(n, oracle_lib):
         assert np.array_equal(pb[i], (yb[3:] - dot * u[i]) / E[i] + (-(kb * kap[i]) / E[i]) * u[i]), i
     assert np.allclose(gb, go, rtol=1e-10, atol=1e-12 * np.abs(go).max())
     assert np.array_equal(gb == 0, go == 0)
+
+
+@pytest.mark.parametrize("n,steps,K", [(1, 1, 64), (3, 7, 64), (11, 40, 3), (609, 5, 2), (6090, 3, 64)])
+def test_records_per_step_match_the_oracle(oracle_lib, n, steps, K):
+    """One chain and one step up to more chains than one block per SM takes, chunks of one step, and
+    checkpoints closer and wider than the steps: steps, end states and per-chain gradients bit for bit."""
+    import torch
+
+    from paper_1410_5323_gb300.adjoint import Adjoint
+    import paper_1410_5323_gb300 as crp
+
+    g = I.kolmogorov_grid(18, 0.25 * I.MPC, 2, 8, 1e-13, 3).astype(np.float32)
+    rng = np.random.default_rng(n)
+    x0 = rng.uniform(-3, 3, (n, 3)) * I.MPC
+    p0 = I.isotropic_directions(n, rng) * 10 ** rng.uniform(18.5, 20, n)[:, None]
+    Z = rng.integers(1, 27, n).astype(np.int32)
+    bar = rng.standard_normal((n, 3))
+    a = Adjoint(crp.Field(g, 0.25 * I.MPC), n, steps, K)
+    _, uT = a.forward(torch.from_numpy(x0), torch.from_numpy(p0), torch.from_numpy(Z), 1e-4, I.KPC, I.MPC)
+    _, pb, xb = a.backward(torch.from_numpy(bar), g.shape)
+    h, uT, pb, xb = (v.cpu().numpy() for v in (a.steps(), uT, pb, xb))
+    E, u, kap = _init(p0, Z)
+    of = O.OracleField(g, 0.25 * I.MPC)
+    for i in np.unique(np.linspace(0, n - 1, min(n, 12)).astype(int)):
+        y0 = np.concatenate([x0[i], u[i]])
+        ho, yT = O.record_steps(of, kap[i], y0, 1e-4, I.KPC, I.MPC, steps)
+        assert np.array_equal(h[:, i], ho) and np.array_equal(uT[i], yT[3:]), i
+        yb, kb = O.adjoint(of, kap[i], y0, h[:, i], np.concatenate([np.zeros(3), bar[i]]))
+        assert np.array_equal(xb[i], yb[:3]), i
+        dot = (u[i, 0] * yb[3] + u[i, 1] * yb[4]) + u[i, 2] * yb[5]
+        assert np.array_equal(pb[i], (yb[3:] - dot * u[i]) / E[i] + (-(kb * kap[i]) / E[i]) * u[i]), i
