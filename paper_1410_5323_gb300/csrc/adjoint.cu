@@ -675,7 +675,7 @@ int adj_record(const FieldDev& F, const double* y0, const double* kappa, double 
     const int per_warp = (int)std::max(1ll, std::min<long long>(kTeams, (n + 4 * sms - 1) / (4 * sms)));
     const long long warps = (n + per_warp - 1) / per_warp;
     // up to one block per SM: shared memory that a second one finds no room for spreads them
-    const int shm = warps <= 4 * sms ? 116 * 1024 : 0;
+    const int shm = warps <= 4 * sms ? kOnePerSmBytes : 0;
     if (shm) {
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, shm);
         if (e != cudaSuccess) return (int)e;

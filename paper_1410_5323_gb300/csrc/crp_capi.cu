@@ -437,6 +437,7 @@ struct Plan {
     int team_grid = 0, team_block = 0;   // three-lane kernel: blocks (0: not launched), threads per block
     int team_launches = 0;
     int lane_launches = 2;               // launches of the one-lane kernel before those
+    int spread_launches = 0;             // launches of the precision form with one block per SM after those
 };
 
 }  // namespace
@@ -1415,8 +1416,15 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
     const long long lanes = (long long)P.grid * block;
     // Without tables there are no secondaries and one launch does; with them the second takes those
     // that the first left (all, if they wait for it).
-    P.team_grid = P.team_block = P.team_launches = 0;
+    P.team_grid = P.team_block = P.team_launches = P.spread_launches = 0;
     P.lane_launches = mixed && !s->tables ? 1 : 2;
+    // Precision form: lists that fit one block per SM go to launches of that shape, which deal the
+    // particles out evenly (1024 protons over 100 Mpc: 764 -> 568 us; 19 000 over 50 Mpc: 1076 -> 961 us).
+    const long long one_layer = (long long)sms * block;
+    if (mixed && prm->blocks_per_sm <= 0) {
+        P.spread_launches = s->tables ? 2 : 1;
+        P.lane_launches = s->capacity <= one_layer ? 0 : (s->tables && pickup == CRP_PICKUP_OFF ? 2 : 1);
+    }
     if (team) {
         int occ = prm->blocks_per_sm;
         if (occ <= 0 && (propagate_team_occupancy(s->mod, p2, block, &occ) != 0 || occ < 1)) occ = 1;
@@ -1447,8 +1455,9 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
     // on the 10^6-nuclei workload), 1 in the FP64 form; results do not depend on it
     a.cadence = prm->cadence > 0 ? prm->cadence : (prm->form == CRP_FORM_MIXED ? 2 : 1);
     a.pickup = take_up;
+    a.spread = 0;
     a.drain = team ? 1 : 0;
-    a.min_work = team ? lanes : -1;
+    a.min_work = team ? lanes : (P.spread_launches ? one_layer : -1);
     a.taken = team ? s->taken : nullptr;
     a.back = team ? 1 : 0;
     a.lists[0] = s->lists[0];
@@ -1502,6 +1511,16 @@ int enqueue(crp_sim* s, const Plan& P, cudaStream_t st) {
         k_swap<<<1, tidy ? 1024 : 1, 0, st>>>(s->ctr, s->capacity, a.min_work, tidy ? s->lists[0] : nullptr, s->lists[1]);
         CRP_CUDA(cudaGetLastError());
     }
+    for (int gen = 0; gen < P.spread_launches; ++gen) {
+        PropArgs t = a;
+        t.spread = 1;
+        t.min_work = -1;
+        if (gen > 0) t.pickup = 0;      // nucleons: they release nothing
+        int e = launch_propagate_mixed(t, P.layout, P.mod, P.p2, std::max(1, s->sms), P.block, st);
+        if (e) return cuda_fail((cudaError_t)e, "propagate kernel launch");
+        k_swap<<<1, tidy ? 1024 : 1, 0, st>>>(s->ctr, s->capacity, -1, tidy ? s->lists[0] : nullptr, s->lists[1]);
+        CRP_CUDA(cudaGetLastError());
+    }
     for (int gen = 0; gen < P.team_launches; ++gen) {
         // one that drains if the particles may not fit one block per SM, one for what is left, and one
         // for the secondaries that this released late (nucleons, which release nothing)
@@ -1552,7 +1571,7 @@ bool same_plan(const Plan& x, const Plan& y) {
            x.block == y.block && x.order == y.order && x.mixed == y.mixed && x.n_buckets == y.n_buckets &&
            x.p2 == y.p2 && x.team_grid == y.team_grid && x.team_block == y.team_block &&
            x.team_launches == y.team_launches &&
-           x.lane_launches == y.lane_launches && x.layout == y.layout && x.mod == y.mod;
+           x.lane_launches == y.lane_launches && x.spread_launches == y.spread_launches && x.layout == y.layout && x.mod == y.mod;
 }
 
 }  // namespace

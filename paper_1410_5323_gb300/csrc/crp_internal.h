@@ -103,6 +103,8 @@ struct PropArgs {
     int32_t cadence;
     int32_t pickup;                  // take secondaries pushed during the launch: 1 once the list has run
                                      // out, 2 before the rest of the list
+    int32_t spread;                  // precision form: one block per SM, particles evenly over its warps
+    int32_t pad2_;
     int32_t drain;                   // once the list has run out (and, in the three-lane kernel, at most
     int32_t back;                    // drain_at particles are left), hand active particles to the next launch
     long long drain_at;              // back: lists that a launch of this call filled are taken from their end
@@ -139,6 +141,8 @@ int launch_propagate_fp64(const PropArgs& a, int layout, int mod, int p2, int gr
 int propagate_fp64_occupancy(int layout, int mod, int p2, int block, int* blocks_per_sm);
 // Three lanes per particle (propagate_team.cu); reads FP64 node copies only.
 constexpr int kTeamsPerWarp = 10;
+// Dynamic shared memory of launches with one block per SM: more than half of an SM's 227 KB.
+constexpr int kOnePerSmBytes = 116 * 1024;
 int launch_propagate_team(const PropArgs& a, int mod, int p2, int grid, int block, int one_per_sm, void* stream);
 int propagate_team_occupancy(int mod, int p2, int block, int* blocks_per_sm);
 int launch_propagate_mixed(const PropArgs& a, int layout, int mod, int p2, int grid, int block, void* stream);

@@ -22,6 +22,8 @@
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
+
 #include "crp_internal.h"
 #include "crp_math.cuh"
 #include "crp_sched.cuh"
@@ -348,8 +350,13 @@ __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* s
     Counters* C = a.ctr;
     const WorkList work = work_list(a);
     const int pushes = 1 - work.L;
+    if ((long long)(work.n_work - work.head0) <= a.min_work) return;
     const float INF = __int_as_float(0x7f800000);
     const SimState& S = a.st;
+    // a batch that can't fill one block per SM: evenly over the warps, since the lanes of a warp wait
+    // for each other's cells and run each other's branches
+    const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
+    const int quota = a.spread ? (int)min(32ull, (work.n_work - work.head0 + warps - 1) / warps) : 32;
     const double tol2 = a.tol * a.tol;
     const float inv_tol2 = (float)(1.0 / tol2);
     // Guard band of the accept decision: an FP32 squared norm at most tol2_lo (at least
@@ -419,7 +426,7 @@ __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* s
         int popped = -1, resumed = 0;
         if (PICK && sched_look<32>(a, dry, turn)) popped = sched_pick(a, pushes, slot < 0, lane, bits, resumed);
         if (!dry) {
-            const int p = sched_pop(a, work, slot < 0 && popped < 0, lane, bits, dry, resumed);
+            const int p = sched_pop(a, work, slot < 0 && popped < 0 && lane < quota, lane, bits, dry, resumed);
             if (p >= 0) popped = p;
         }
         if (popped >= 0) {
@@ -807,10 +814,13 @@ static int mixed_carveout_pct(int grid, size_t shm_per_block) {
 
 int launch_propagate_mixed(const PropArgs& a, int layout, int mod, int p2, int grid, int block, void* stream) {
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const size_t shm = mixed_smem(mod, block);
-    const int pct = mixed_carveout_pct(grid, shm);
+    // spread: shared memory that only one block of an SM finds room for
+    const size_t shm = a.spread ? std::max(mixed_smem(mod, block), (size_t)kOnePerSmBytes) : mixed_smem(mod, block);
+    const int pct = a.spread ? -1 : mixed_carveout_pct(grid, shm);
     return with_mixed_kernel(layout, mod, p2, a.pickup, [&](void (*k)(const PropArgs)) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+        if (e == cudaSuccess && a.spread)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
         if (e != cudaSuccess) return (int)e;
         k<<<grid, block, shm, st>>>(a);
         return (int)cudaGetLastError();

@@ -32,8 +32,6 @@ namespace {
 
 using namespace team;
 
-constexpr int kOnePerSmBytes = 116 * 1024;   // more than half of an SM's 227 KB
-
 template <bool M, bool P2>
 __global__ void __launch_bounds__(256, M ? 1 : 2) k_propagate_fp64_team(const PropArgs a) {
     CRP_COUNT_RUN();

@@ -76,3 +76,24 @@ def test_options_small_batch(oracle_lib):
     grids = [_grid(18, 13), _grid(18, 14)]
     _same(grids, p, None, 1e-4, I.KPC, I.MPC, 6 * I.MPC, origin=(0.3 * I.MPC, -0.1 * I.MPC, 0.0), mods=mods,
           mod_spacing=0.6 * I.MPC, box=box)
+
+
+@pytest.mark.parametrize("tables", [False, True])
+@pytest.mark.parametrize("n,spare", [(1, 0), (40, 0), (19455, 1), (19457, 0), (300, 40_000)])
+def test_precision_form_spread_over_the_device(n, spare, tables):
+    """The precision form's launches of one block per SM (small simulations, small lists of large ones,
+    and lists just above the limit) against its launches of a fixed shape: the same particles."""
+    import paper_1410_5323_gb300 as crp
+
+    p = I.make_particles(n, 21, species=MIX, energy=("power", 1e18, 10 ** 20.5, 2.0))
+    f = crp.Field(_grid(16, 8), 0.25 * I.MPC)
+    t = crp.Tables(I.constant_rate_tables(1 / (300 * I.MPC), 1 / (20 * I.MPC))) if tables else None
+    got = []
+    for per_sm in (0, 2):
+        sim = crp.Simulation([f], t, seed=4, capacity=(2 * n + 50 if tables else n) + spare)
+        sim.inject(p)
+        sim.propagate(1e-4, I.KPC, I.MPC, 2 * I.MPC, form=crp.FORM_MIXED, blocks_per_sm=per_sm)
+        assert sim.sync(60.0) == 0
+        got.append(by_uid(sim.state()))
+    for k in got[0]:
+        assert np.array_equal(got[0][k], got[1][k], equal_nan=got[0][k].dtype.kind == "f"), k
