@@ -609,6 +609,7 @@ int crp_field_create(const void* grid, int32_t dtype, int32_t is_device, int32_t
     d.spacing = spacing_m;
     d.ox = origin_m[0]; d.oy = origin_m[1]; d.oz = origin_m[2];
     d.oix = d.ox * d.inv_spacing; d.oiy = d.oy * d.inv_spacing; d.oiz = d.oz * d.inv_spacing;
+    d.ox_f = (float)d.ox; d.oy_f = (float)d.oy; d.oz_f = (float)d.oz;
     d.scale = (dtype == CRP_DTYPE_BF16 || dtype == CRP_DTYPE_F16) ? (double)scale : 1.0;
     d.mod = nullptr;
     *out = f;
@@ -1470,6 +1471,8 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
         a.box_hi[c] = s->box_origin[c] + s->box_size[c];
         a.box_len[c] = s->box_size[c];
         a.box_inv[c] = s->boundary == CRP_BOUNDARY_REFLECT ? 1.0 / s->box_size[c] : 0.0;
+        a.box_lo_f[c] = (float)a.box_lo[c];
+        a.box_hi_f[c] = (float)a.box_hi[c];
     }
     return CRP_OK;
 }

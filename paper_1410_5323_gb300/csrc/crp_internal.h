@@ -25,6 +25,8 @@ struct FieldDev {
     double spacing;
     double ox, oy, oz;
     double oix, oiy, oiz;    // origin * (1/spacing), rounded once
+    float ox_f, oy_f, oz_f;  // origin in FP32
+    float pad2_;
     double scale;            // BF16/F16 multiplier (1 otherwise)
     // Modulation grid (Sec. 3.2 modulated grids): B(x) = M(x) b(x) with M a scalar FP32
     // periodic grid, node (i,j,k) at (i*mny + j)*mnz + k; nullptr when the field has none.
@@ -117,6 +119,7 @@ struct PropArgs {
     int32_t boundary;
     int32_t pad_;
     double box_lo[3], box_hi[3], box_len[3], box_inv[3];
+    float box_lo_f[3], box_hi_f[3];
 };
 
 // Launchers (defined in the kernel translation units).
