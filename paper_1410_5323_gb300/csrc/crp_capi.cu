@@ -1454,7 +1454,12 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
     a.capacity = s->capacity;
     // default cadence: 2 attempts between refill checks in the precision form (measured +1.5 %
     // on the 10^6-nuclei workload), 1 in the FP64 form; results do not depend on it
-    a.cadence = prm->cadence > 0 ? prm->cadence : (prm->form == CRP_FORM_MIXED ? 2 : 1);
+    // Default cadence, attempts between refill checks (results do not depend on it). A refill is ~35 FP64
+    // instructions and a round trip for the whole warp, so the precision form lets lanes idle a little
+    // to fill several at once: 8 without secondaries (sky map of 10^6 sources 1.75 ms at 2, 1.57 at 8;
+    // 10^6 p/Fe on 512^3 40.5 and 39.7; 64 x 128^3 fields 38.2 and 37.2), 2 where idle lanes also take
+    // secondaries up (10^6 nuclei 63.9 ms at 2, 71.7 at 4); 1 in the FP64 form.
+    a.cadence = prm->cadence > 0 ? prm->cadence : (!mixed ? 1 : (take_up ? 2 : 8));
     a.pickup = take_up;
     a.spread = 0;
     a.drain = team ? 1 : 0;
