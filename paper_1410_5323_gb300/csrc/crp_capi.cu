@@ -204,8 +204,9 @@ __global__ void k_set_used(Counters* C, unsigned long long n_used, unsigned long
 }
 
 // ---- propagate bookkeeping ----------------------------------------------------------------
-__global__ void k_prepare(Counters* C) {
+__global__ void k_prepare(Counters* C, int pickup) {
     CRP_COUNT_RUN();
+    if (!pickup) C->tidy = 0;
     C->count[0] = 0;
     C->count[1] = 0;
     C->head[0] = 0;
@@ -215,6 +216,20 @@ __global__ void k_prepare(Counters* C) {
     C->pushed = 0;
     C->head0 = 0;
     C->left = 0;
+}
+
+// Puts -1 (nothing published) into both work lists if an earlier call left entries in them; l0 is
+// NULL in calls that take nothing up. The state of the lists is kept on the device, so that calls
+// replayed from a graph, in any order, find it as it is.
+__device__ __forceinline__ void clear_lists(int32_t* l0, int32_t* l1, long long len, const Counters* C) {
+    if (!l0 || *(volatile const int*)&C->tidy) return;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < len; i += (long long)gridDim.x * blockDim.x)
+        l0[i] = l1[i] = -1;
+}
+
+__global__ void k_clear_lists(int32_t* l0, int32_t* l1, long long len, const Counters* C) {
+    CRP_COUNT_RUN();
+    clear_lists(l0, l1, len, C);
 }
 
 // ---- work list in order of expected cost (longest first) ------------------------------
@@ -236,8 +251,9 @@ __device__ __forceinline__ int sort_key(double E, int Z, int gid, int grid_major
 __global__ void k_cost_hist(const int32_t* __restrict__ status, const double* __restrict__ E,
                             const int32_t* __restrict__ Zc, const int32_t* __restrict__ gid,
                             int grid_major, int n_buckets, int use_shared,
-                            unsigned* __restrict__ hist, const Counters* C) {
+                            unsigned* __restrict__ hist, const Counters* C, int32_t* l0, int32_t* l1, long long len) {
     CRP_COUNT_RUN();
+    clear_lists(l0, l1, len, C);
     extern __shared__ unsigned sh[];
     if (use_shared) {
         for (int b = threadIdx.x; b < n_buckets; b += blockDim.x) sh[b] = 0;
@@ -340,6 +356,7 @@ __global__ void k_swap(Counters* C, long long capacity, long long min_work, int3
     CRP_COUNT_RUN();
     const int from = C->cur;
     const long long n = (long long)C->count[from];
+    if (l0 && threadIdx.x == 0) C->tidy = 1;
     if (n - (long long)C->head0 <= min_work) return;
     if (l0) {
         int32_t* l = from ? l1 : l0;
@@ -474,8 +491,8 @@ struct crp_sim {
     int32_t* lists[2] = {nullptr, nullptr};
     int32_t* done_list = nullptr;
     Counters* ctr = nullptr;
-    bool untidy = false;                // the work lists may hold entries of an earlier call
     int32_t* taken = nullptr;           // accepted steps of this call, for particles handed between launches
+                                        // (FP64 form)
     unsigned* sort_scratch = nullptr;   // [hist n_buckets][offsets n_buckets]
     cudaStream_t last = nullptr;
     cudaGraph_t loop_graph = nullptr;   // crp_propagate_loop, cached for one plan
@@ -505,6 +522,13 @@ int alloc_state(SimState& S, long long cap) {
         }
     }
     return CRP_OK;
+}
+
+// Entries a work list can hold. A launch pushes each slot at most once as a new secondary and once as
+// a particle handed on to the next launch, the latter at most one per thread; a particle that is in
+// the list both times was taken up in between.
+long long list_length(const crp_sim* s, long long capacity) {
+    return capacity + std::min(capacity, (long long)std::max(1, s->sms) * kThreadsPerSm);
 }
 
 int sync_stream(crp_sim* s) {
@@ -753,12 +777,10 @@ int crp_sim_create(const crp_field* const* fields, int32_t n_fields, const crp_t
     if (rc == CRP_OK) e = dev_malloc(&s->d_fields, sizeof(FieldDev) * n_fields);
     if (rc == CRP_OK && e == cudaSuccess)
         e = cudaMemcpy(s->d_fields, s->host_fields.data(), sizeof(FieldDev) * n_fields, cudaMemcpyHostToDevice);
-    if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->lists[0], sizeof(int32_t) * capacity);
-    if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->lists[1], sizeof(int32_t) * capacity);
+    if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->lists[0], sizeof(int32_t) * list_length(s, capacity));
+    if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->lists[1], sizeof(int32_t) * list_length(s, capacity));
     if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->done_list, sizeof(int32_t) * capacity);
-    if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->taken, sizeof(int32_t) * capacity);
-    for (int k = 0; k < 2; ++k)   // no entry published
-        if (rc == CRP_OK && e == cudaSuccess) e = cudaMemset(s->lists[k], 0xff, sizeof(int32_t) * capacity);
+    if (rc == CRP_OK && e == cudaSuccess && layout == LAYOUT_F64X4) e = dev_malloc(&s->taken, sizeof(int32_t) * capacity);
     if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->ctr, sizeof(Counters));
     if (rc == CRP_OK && e == cudaSuccess) e = cudaMemset(s->ctr, 0, sizeof(Counters));
     const size_t sort_bytes = 2 * (size_t)kBuckets * n_fields * sizeof(unsigned);
@@ -838,12 +860,11 @@ int crp_sim_reserve(crp_sim* s, int64_t capacity) {
     rc = alloc_state(ns, capacity);
     if (rc) return rc;
     int32_t *l0 = nullptr, *l1 = nullptr, *dl = nullptr, *tk = nullptr;
-    cudaError_t e = dev_malloc(&l0, sizeof(int32_t) * capacity);
-    if (e == cudaSuccess) e = dev_malloc(&tk, sizeof(int32_t) * capacity);
-    if (e == cudaSuccess) e = dev_malloc(&l1, sizeof(int32_t) * capacity);
+    cudaError_t e = dev_malloc(&l0, sizeof(int32_t) * list_length(s, capacity));
+    if (e == cudaSuccess) e = dev_malloc(&l1, sizeof(int32_t) * list_length(s, capacity));
     if (e == cudaSuccess) e = dev_malloc(&dl, sizeof(int32_t) * capacity);
-    if (e == cudaSuccess) e = cudaMemset(l0, 0xff, sizeof(int32_t) * capacity);
-    if (e == cudaSuccess) e = cudaMemset(l1, 0xff, sizeof(int32_t) * capacity);
+    if (e == cudaSuccess && s->taken) e = dev_malloc(&tk, sizeof(int32_t) * capacity);
+    if (e == cudaSuccess) e = cudaMemset(&s->ctr->tidy, 0, sizeof(int));   // new lists
     for (int c = 0; c < CRP_N_COLS && e == cudaSuccess; ++c)
         e = cudaMemcpy(*col_ptr(ns, c), *col_ptr(s->st, c), (size_t)h.n_used * kCols[c].size,
                        cudaMemcpyDeviceToDevice);
@@ -861,9 +882,8 @@ int crp_sim_reserve(crp_sim* s, int64_t capacity) {
     cudaFree(s->lists[0]);
     cudaFree(s->lists[1]);
     cudaFree(s->done_list);
-    cudaFree(s->taken);
+    if (s->taken) cudaFree(s->taken);
     s->taken = tk;
-    s->untidy = false;
     s->st = ns;
     s->lists[0] = l0;
     s->lists[1] = l1;
@@ -1374,6 +1394,8 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
         if (rc) return rc;
         fields = s->d_fields64;
         layout = LAYOUT_F64X4;
+        // without room for it particles stay in the launch that took them
+        if (!s->taken && dev_malloc(&s->taken, sizeof(int32_t) * s->capacity) != cudaSuccess) cudaGetLastError();
     }
     if (prm->grid_layout != CRP_GRID_AUTO && prm->grid_layout != CRP_GRID_NODES &&
         prm->grid_layout != CRP_GRID_CELLS)
@@ -1409,11 +1431,12 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
     }
     const int sms = s->sms > 0 ? s->sms : 1;
     PropArgs& a = P.a;
-    P.grid = sms * bps;
     // FP64: the one-lane kernel for what fills its lanes, the three-lane kernel for the rest
     // (simulations that can't fill them launch only that). PICKUP_ON asks for the one-lane
     // kernel's own handling of secondaries.
     const bool team = !mixed && pickup != CRP_PICKUP_ON && layout == LAYOUT_F64X4;
+    if (team) bps = std::min(bps, kThreadsPerSm / block);   // no more than run at once: list_length
+    P.grid = sms * bps;
     const long long lanes = (long long)P.grid * block;
     // Without tables there are no secondaries and one launch does; with them the second takes those
     // that the first left (all, if they wait for it).
@@ -1429,7 +1452,7 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
     if (team) {
         int occ = prm->blocks_per_sm;
         if (occ <= 0 && (propagate_team_occupancy(s->mod, p2, block, &occ) != 0 || occ < 1)) occ = 1;
-        P.team_grid = sms * occ;
+        P.team_grid = sms * std::min(occ, kThreadsPerSm / block);
         P.team_block = block;
         P.lane_launches = s->capacity <= lanes ? 0 : (s->tables && pickup == CRP_PICKUP_OFF ? 2 : 1);
         // what one block per SM takes up needs no launch that drains
@@ -1452,8 +1475,6 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
     a.seed = s->seed;
     a.max_steps = prm->max_steps;
     a.capacity = s->capacity;
-    // default cadence: 2 attempts between refill checks in the precision form (measured +1.5 %
-    // on the 10^6-nuclei workload), 1 in the FP64 form; results do not depend on it
     // Default cadence, attempts between refill checks (results do not depend on it). A refill is ~35 FP64
     // instructions and a round trip for the whole warp, so the precision form lets lanes idle a little
     // to fill several at once: 8 without secondaries (sky map of 10^6 sources 1.75 ms at 2, 1.57 at 8;
@@ -1462,7 +1483,7 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
     a.cadence = prm->cadence > 0 ? prm->cadence : (!mixed ? 1 : (take_up ? 2 : 8));
     a.pickup = take_up;
     a.spread = 0;
-    a.drain = team ? 1 : 0;
+    a.drain = team && s->taken ? 1 : 0;
     a.min_work = team ? lanes : (P.spread_launches ? one_layer : -1);
     a.taken = team ? s->taken : nullptr;
     a.back = team ? 1 : 0;
@@ -1485,10 +1506,14 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
 // The launch sequence of one propagate call (no host synchronisation; capturable).
 int enqueue(crp_sim* s, const Plan& P, cudaStream_t st) {
     PropArgs a = P.a;
-    k_prepare<<<1, 1, 0, st>>>(s->ctr);
+    k_prepare<<<1, 1, 0, st>>>(s->ctr, a.pickup);
     CRP_CUDA(cudaGetLastError());
     const int sgrid = (s->sms > 0 ? s->sms : 1) * 4;
+    const bool tidy = a.pickup != 0;
+    int32_t* l0 = tidy ? s->lists[0] : nullptr;
+    const long long len = list_length(s, s->capacity);
     if (P.order == CRP_ORDER_SLOT) {
+        if (tidy) k_clear_lists<<<sgrid, 256, 0, st>>>(l0, s->lists[1], len, s->ctr);
         k_build_worklist<<<sgrid, 256, 0, st>>>(s->st.status, s->lists[0], s->ctr);
     } else {
         const int grid_major = P.order == CRP_ORDER_GRID ? 1 : 0;
@@ -1500,7 +1525,7 @@ int enqueue(crp_sim* s, const Plan& P, cudaStream_t st) {
         const size_t shm = (size_t)P.n_buckets * sizeof(unsigned);
         k_cost_hist<<<sgrid, 256, shm <= 48 * 1024 ? shm : 0, st>>>(
             s->st.status, s->st.E, s->st.Z, s->st.grid_id, grid_major, P.n_buckets,
-            shm <= 48 * 1024 ? 1 : 0, hist, s->ctr);
+            shm <= 48 * 1024 ? 1 : 0, hist, s->ctr, l0, s->lists[1], len);
         k_cost_scan<<<1, 1024, 0, st>>>(hist, offs, P.n_buckets, s->ctr);
         k_cost_scatter<<<sgrid, 256, 0, st>>>(s->st.status, s->st.E, s->st.Z, s->st.grid_id,
                                               grid_major, offs, s->lists[0], s->ctr);
@@ -1511,12 +1536,11 @@ int enqueue(crp_sim* s, const Plan& P, cudaStream_t st) {
     // launches finish the call. With the three-lane kernel a one-lane launch hands its active
     // particles on when its list has run out, to the next list with the secondaries, and the
     // three-lane launches finish them.
-    const bool tidy = a.pickup != 0;
     for (int gen = 0; gen < P.lane_launches; ++gen) {
         int e = P.mixed ? launch_propagate_mixed(a, P.layout, P.mod, P.p2, P.grid, P.block, st)
                         : launch_propagate_fp64(a, P.layout, P.mod, P.p2, P.grid, P.block, st);
         if (e) return cuda_fail((cudaError_t)e, "propagate kernel launch");
-        k_swap<<<1, tidy ? 1024 : 1, 0, st>>>(s->ctr, s->capacity, a.min_work, tidy ? s->lists[0] : nullptr, s->lists[1]);
+        k_swap<<<1, tidy ? 1024 : 1, 0, st>>>(s->ctr, s->capacity, a.min_work, l0, s->lists[1]);
         CRP_CUDA(cudaGetLastError());
     }
     for (int gen = 0; gen < P.spread_launches; ++gen) {
@@ -1526,34 +1550,22 @@ int enqueue(crp_sim* s, const Plan& P, cudaStream_t st) {
         if (gen > 0) t.pickup = 0;      // nucleons: they release nothing
         int e = launch_propagate_mixed(t, P.layout, P.mod, P.p2, std::max(1, s->sms), P.block, st);
         if (e) return cuda_fail((cudaError_t)e, "propagate kernel launch");
-        k_swap<<<1, tidy ? 1024 : 1, 0, st>>>(s->ctr, s->capacity, -1, tidy ? s->lists[0] : nullptr, s->lists[1]);
+        k_swap<<<1, tidy ? 1024 : 1, 0, st>>>(s->ctr, s->capacity, -1, l0, s->lists[1]);
         CRP_CUDA(cudaGetLastError());
     }
     for (int gen = 0; gen < P.team_launches; ++gen) {
         // one that drains if the particles may not fit one block per SM, one for what is left, and one
         // for the secondaries that this released late (nucleons, which release nothing)
         PropArgs t = a;
-        t.drain = gen == 0 && s->capacity > a.drain_at ? 1 : 0;
+        t.drain = a.drain && gen == 0 && s->capacity > a.drain_at ? 1 : 0;
         t.min_work = t.drain ? a.drain_at : -1;
         if (gen == P.team_launches - 1) t.pickup = 0;
         int e = launch_propagate_team(t, P.mod, P.p2, t.drain ? P.team_grid : std::max(1, s->sms), P.team_block,
                                       t.drain ? 0 : 1, st);
         if (e) return cuda_fail((cudaError_t)e, "propagate kernel launch");
-        k_swap<<<1, tidy ? 1024 : 1, 0, st>>>(s->ctr, s->capacity, t.min_work, tidy ? s->lists[0] : nullptr, s->lists[1]);
+        k_swap<<<1, tidy ? 1024 : 1, 0, st>>>(s->ctr, s->capacity, t.min_work, l0, s->lists[1]);
         CRP_CUDA(cudaGetLastError());
     }
-    return CRP_OK;
-}
-
-// Before a call's launches on `st`: clears lists that a call without pick-ups left as they were.
-int tidy_lists(crp_sim* s, const Plan& P, cudaStream_t st) {
-    if (!P.a.pickup) {
-        s->untidy = true;
-        return CRP_OK;
-    }
-    for (int k = 0; k < 2 && s->untidy; ++k)
-        CRP_CUDA(cudaMemsetAsync(s->lists[k], 0xff, sizeof(int32_t) * s->capacity, st));
-    s->untidy = false;
     return CRP_OK;
 }
 
@@ -1593,8 +1605,7 @@ int crp_propagate(crp_sim* s, const crp_params* prm, double tol, double hmin, do
     int rc = make_plan(s, prm, tol, hmin, hmax, dmax, P);
     if (rc) return rc;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    rc = tidy_lists(s, P, st);
-    if (!rc) rc = enqueue(s, P, st);
+    rc = enqueue(s, P, st);
     if (rc) return rc;
     s->last = st;
     return CRP_OK;
@@ -1650,8 +1661,6 @@ int crp_propagate_loop(crp_sim* s, const crp_params* prm, double tol, double hmi
         s->loop_plan = P;
         s->loop_max_slices = max_slices;
     }
-    rc = tidy_lists(s, P, st);
-    if (rc) return rc;
     CRP_CUDA(cudaGraphLaunch(s->loop_exec, st));
     s->last = st;
     return CRP_OK;
@@ -1879,7 +1888,7 @@ extern "C" int crp_propagate_noalloc(const void* grid, int32_t nx, int32_t ny, i
     k_inject_init<<<grid_for(n, 256, 4096), 256, 0, st>>>(S, 0, n, 1, 0, 0ull, 1, 0, 0, 0, seed,
                                                           done, ctr);
     CRP_CUDA(cudaGetLastError());
-    k_prepare<<<1, 1, 0, st>>>(ctr);
+    k_prepare<<<1, 1, 0, st>>>(ctr, 0);
     CRP_CUDA(cudaGetLastError());
     k_build_worklist<<<sms * 4, 256, 0, st>>>(S.status, l0, ctr);
     CRP_CUDA(cudaGetLastError());

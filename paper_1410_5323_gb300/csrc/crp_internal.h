@@ -87,7 +87,7 @@ struct Counters {
     unsigned int status_bits;
     int cur;                         // work list (0 or 1) that the next propagate launch takes
     int pushed;                      // that list was filled by a propagate launch of this call
-    int pad_;
+    int tidy;                        // the work lists hold no entry of an earlier call (calls with pick-up keep them so)
     unsigned long long head0;        // first entry of that list (earlier ones were picked up when pushed)
     unsigned long long left;         // entries of the list whose particle the current launch has stored
 };
@@ -144,6 +144,7 @@ int launch_propagate_fp64(const PropArgs& a, int layout, int mod, int p2, int gr
 int propagate_fp64_occupancy(int layout, int mod, int p2, int block, int* blocks_per_sm);
 // Three lanes per particle (propagate_team.cu); reads FP64 node copies only.
 constexpr int kTeamsPerWarp = 10;
+constexpr int kThreadsPerSm = 2048;      // resident threads of an SM
 // Dynamic shared memory of launches with one block per SM: more than half of an SM's 227 KB.
 constexpr int kOnePerSmBytes = 116 * 1024;
 int launch_propagate_team(const PropArgs& a, int mod, int p2, int grid, int block, int one_per_sm, void* stream);

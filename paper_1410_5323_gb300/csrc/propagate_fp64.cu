@@ -89,7 +89,7 @@ __global__ void CRP_FP64_BOUNDS k_propagate_fp64(const PropArgs a) {
         // ---- refill idle lanes from the work list (one atomic per warp) ----
         int popped = -1, resumed = 0;
         if (sched_look<4>(a, dry, turn) && !(dry && a.drain))
-            popped = sched_pick(a, pushes, slot < 0, lane, bits, resumed);
+            popped = sched_pick_secondaries(a, pushes, slot < 0, lane, bits);
         if (!dry) {
             const int p = sched_pop(a, work, slot < 0 && popped < 0, lane, bits, dry, resumed);
             if (p >= 0) popped = p;

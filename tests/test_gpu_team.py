@@ -97,3 +97,44 @@ def test_precision_form_spread_over_the_device(n, spare, tables):
         got.append(by_uid(sim.state()))
     for k in got[0]:
         assert np.array_equal(got[0][k], got[1][k], equal_nan=got[0][k].dtype.kind == "f"), k
+
+
+@pytest.mark.parametrize("n", [400, 9000, 60_000])
+def test_no_slot_to_spare(n):
+    """As many slots as the run uses: the lists hold secondaries and particles handed on at once."""
+    import paper_1410_5323_gb300 as crp
+
+    p = I.make_particles(n, 4, species=MIX, energy=("power", 1e18, 10 ** 20.5, 2.0))
+    f, t = crp.Field(_grid(16, 8), 0.25 * I.MPC), crp.Tables(I.constant_rate_tables(0.0, 1 / (2 * I.MPC)))
+    states, capacity = [], 30 * n
+    for _ in range(2):
+        sim = crp.Simulation([f], t, seed=5, capacity=capacity)
+        sim.inject(p)
+        sim.propagate(1e-4, I.KPC, I.MPC, 3 * I.MPC, form=crp.FORM_FP64)
+        assert sim.sync(60.0) == 0
+        capacity = n + sim.counts()["secondaries"]
+        states.append(by_uid(sim.state()))
+    assert capacity > n
+    assert_bit_identical(*states)
+
+
+def test_calls_with_and_without_pickup_on_one_simulation():
+    """Lists that a call without pick-ups left full are cleared before the next one looks into them."""
+    import paper_1410_5323_gb300 as crp
+
+    p = I.make_particles(3000, 12, species=MIX, energy=("power", 1e18, 10 ** 20.5, 2.0))
+    f, t = crp.Field(_grid(16, 9), 0.25 * I.MPC), crp.Tables(I.constant_rate_tables(0.0, 1 / (4 * I.MPC)))
+    for form in (crp.FORM_FP64, crp.FORM_MIXED):
+        states = []
+        for modes in ((1, 1, 1, 1), (1, 0, 2, 0), (0, 1, 0, 2)):
+            sim = crp.Simulation([f], t, seed=6, capacity=56 * 3000)
+            sim.inject(p)
+            for k, mode in enumerate(modes):
+                sim.propagate(1e-4, I.KPC, I.MPC, 8 * I.MPC, form=form, pickup=mode, max_steps=4 if k < 3 else 0,
+                              order=k % 3)
+                if k == 1:
+                    sim.reserve(60 * 3000)
+            assert sim.sync(60.0) == 0
+            states.append(by_uid(sim.state()))
+        for s in states[1:]:
+            assert_bit_identical(states[0], s)
