@@ -107,9 +107,10 @@ struct PropArgs {
                                      // out, 2 before the rest of the list
     int32_t spread;                  // precision form: one block per SM, particles evenly over its warps
     int32_t pad2_;
-    int32_t drain;                   // once the list has run out (and, in the three-lane kernel, at most
-    int32_t back;                    // drain_at particles are left), hand active particles to the next launch
-    long long drain_at;              // back: lists that a launch of this call filled are taken from their end
+    int32_t drain;                   // once the list has run out and at most drain_at particles are left, hand
+                                     // active particles on to the next launch
+    int32_t back;                    // lists that a launch of this call filled are taken from their end
+    long long drain_at;
     long long min_work;              // a launch leaves lists of at most this many entries to the next one
     int32_t* taken;                  // per slot: accepted steps of this call so far (drained particles); may be NULL
     int32_t* lists[2];               // list Counters::cur is processed, secondaries are pushed to the other

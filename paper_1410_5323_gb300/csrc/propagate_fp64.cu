@@ -6,7 +6,7 @@
 // a new step stay converged. Idle lanes are refilled from a global work counter with one
 // warp-aggregated atomic (ballot + popc); finished particles are appended to the done
 // list; secondaries reserve a slot atomically and go to the other work list, from which
-// idle lanes of this launch or the next launch take them. When the work list has run out
+// idle lanes of this launch or the next launch take them. When the list has run out and lanes empty,
 // the particles still active go to the other list too, for the kernel that has three lanes
 // per particle (propagate_team.cu): a trajectory's time here is 23 us an attempt at the least.
 //
@@ -81,14 +81,15 @@ __global__ void CRP_FP64_BOUNDS k_propagate_fp64(const PropArgs a) {
             const unsigned long long d = atomicAdd(&C->n_done, 1ull);
             a.done_list[d] = slot;
         }
+        if (a.drain) atomicAdd(&C->left, 1ull);
         slot = -1;
     };
 
-    bool dry = false;
+    bool dry = false, drain = false;
     for (unsigned turn = 0;; ++turn) {
         // ---- refill idle lanes from the work list (one atomic per warp) ----
         int popped = -1, resumed = 0;
-        if (sched_look<4>(a, dry, turn) && !(dry && a.drain))
+        if (!drain && sched_look<4>(a, dry, turn))
             popped = sched_pick_secondaries(a, pushes, slot < 0, lane, bits);
         if (!dry) {
             const int p = sched_pop(a, work, slot < 0 && popped < 0, lane, bits, dry, resumed);
@@ -98,8 +99,13 @@ __global__ void CRP_FP64_BOUNDS k_propagate_fp64(const PropArgs a) {
                 head = __shfl_sync(kFull, head, 0);
                 dry = dry || head >= work.n_work;
             }
+        } else if (a.drain && !drain && turn % 8 == 7) {   // few enough for the three-lane kernel?
+            long long left = lane == 0 ? (long long)(work.n_work - work.head0 + ld_volatile(&C->head[pushes]) -
+                                                     ld_volatile(&C->left)) : 0ll;
+            left = __shfl_sync(kFull, left, 0);
+            drain = left <= a.drain_at;
         }
-        if (a.drain && dry && popped < 0 && slot >= 0 && new_step) {   // the next launch resumes it here
+        if (drain && popped < 0 && slot >= 0 && new_step) {   // the next launch resumes it here
             const int32_t q = slot;
             a.taken[q] = (int32_t)taken;
             store(CRP_STATUS_ACTIVE_);
