@@ -1227,12 +1227,16 @@ int crp_lens_create(int32_t n_pix, int32_t n_mat, const int64_t* row_ptr, const 
     L->plain = special ? 0 : 1;
     // Lanes per row for one map: fewer lanes fold fewer partial sums (FP64 additions of the whole
     // warp), so as few as still give every sub-partition ten warps, and no more than a row's 4-entry
-    // vectors. nside 64, 24 bins of 24: 32 lanes 75.8 us, 8 and 4 lanes 68.4 us; nside 64, 5 bins of 8:
-    // 16 lanes 16.4 us, 4 lanes 10.2 us; nside 32, 24 bins of 24: 32, 16, 8 lanes 24.6, 23.9, 31.0 us.
+    // vectors; but where a lane would walk more than 20 vectors, more lanes, which read a longer run at
+    // a time: what counts when the entries come from DRAM. nside 64, 24 bins of 24 (144 vectors a row):
+    // 32 lanes 75.8 us, 8 and 4 lanes 68.4 us; out of L2 80.5, 80.6 and 90.8 us. Of 64 (384 vectors):
+    // 4, 8, 32 lanes 184, 173, 177 us, out of L2 197, 181, 167; of 8 (48): 4 and 8 lanes within 6 %.
+    // nside 64, 5 bins of 8: 16 lanes 16.4 us, 4 lanes 10.2 us; nside 32, 24 bins of 24: 32, 16, 8 lanes
+    // 24.6, 23.9, 31.0 us.
     const double mean = (double)padded / 4.0 / (double)n_pix;
     const long long lanes = 32ll * 10 * 4 * std::max(1, device_sms());
     int g = 4;
-    while (g < 32 && g < mean && (long long)g * n_pix < lanes) g *= 2;
+    while (g < 32 && g < mean && ((long long)g * n_pix < lanes || mean > 20.0 * g)) g *= 2;
     L->group = g;
     *out = L;
     return CRP_OK;
@@ -1538,10 +1542,11 @@ int enqueue(crp_sim* s, const Plan& P, cudaStream_t st) {
     // secondaries, and the three-lane launches finish them.
     for (int gen = 0; gen < P.lane_launches; ++gen) {
         PropArgs l = a;
-        // Handed on once three quarters of the lanes hold a particle: full lanes are worth more than teams
+        // Handed on once half of the lanes hold a particle: full lanes are worth more than teams
         // (10^6 nuclei over 500 Mpc: 7473 ms handing on as soon as the list has run out, 7173 at 6/8 or
-        // less, 7150 without; 60 000 over 100 Mpc: 285 without, 141 at once, 138 at 6/8, 147 at 2/8).
-        if (a.drain) l.drain_at = a.min_work / 4 * 3;
+        // less; 10^6 in a modulated field 5598 at 6/8, 5506 at 4/8, 5513 never; 60 000 over 100 Mpc: 285
+        // without teams, 141 at once, 138 at 6/8, 140 at 4/8, 147 at 2/8).
+        if (a.drain) l.drain_at = a.min_work / 2;
         int e = P.mixed ? launch_propagate_mixed(l, P.layout, P.mod, P.p2, P.grid, P.block, st)
                         : launch_propagate_fp64(l, P.layout, P.mod, P.p2, P.grid, P.block, st);
         if (e) return cuda_fail((cudaError_t)e, "propagate kernel launch");
