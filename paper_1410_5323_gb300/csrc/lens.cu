@@ -197,7 +197,8 @@ __global__ void k_lens_bin(SimState S, const Counters* C, int nside, int n_mat, 
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         if (S.status[i] != CRP_STATUS_DONE_ || S.Z[i] <= 0 || !(S.E[i] > e_min)) continue;
-        // the bin by FP32 rigidity and edges (off by 2^-22 relative) unless R is that near one of them
+        // the bin by FP32 rigidity and edges (off by 2^-22 relative) unless R is that near one of them, or
+        // near the end of the normal FP32 numbers (edges below it read as 0, those above as NaN)
         const float R32 = sky::head_f32(S.E[i]) / (float)S.Z[i];
         int lo = 0, hi = n_mat;              // edges[lo] <= R < edges[hi]
         while (hi - lo > 1) {
@@ -205,9 +206,10 @@ __global__ void k_lens_bin(SimState S, const Counters* C, int nside, int n_mat, 
             if (sky::head_f32(edges[mid]) <= R32) lo = mid; else hi = mid;
         }
         const float below = sky::head_f32(edges[lo]), above = sky::head_f32(edges[lo + 1]);
-        if (!(R32 > below * 1.000002f && R32 < above * 0.999998f)) {
-            if (lo == 0 && R32 < below * 0.999998f) continue;
-            if (lo == n_mat - 1 && R32 > above * 1.000002f) continue;
+        const bool normal = R32 > 1e-37f;
+        if (!(normal && R32 > below * 1.000002f && R32 < above * 0.999998f)) {
+            if (normal && lo == 0 && R32 < below * 0.999998f) continue;
+            if (normal && lo == n_mat - 1 && R32 > above * 1.000002f) continue;
             const double R = S.E[i] / (double)S.Z[i];
             if (!(edges[0] <= R && R < edges[n_mat])) continue;
             lo = 0;

@@ -173,3 +173,31 @@ def test_rows_packed_into_warps_bit_identical(oracle_lib, n_maps):
             val[rng.integers(0, nnz, 40)] = rng.choice(np.float32([0.0, -0.0, 1e-41, -3e-45, np.inf]), 40)
         y = _gpu(crp.Lens(n_pix, rp, col, val), x)
         assert np.array_equal(y, O.lens_apply(n_pix, rp, col, val, x), equal_nan=True)
+
+
+@pytest.mark.parametrize("lo,hi,n_mat", [(1e-46, 1e-36, 40), (1e-40, 1e-38, 3), (1e36, 1e42, 30), (1e-39, 1e39, 7)])
+def test_rigidity_bins_at_the_ends_of_the_float_range(oracle_lib, lo, hi, n_mat):
+    """Edges and rigidities around and beyond the smallest and largest FP32 numbers: exact counts."""
+    import paper_1410_5323_gb300 as crp
+
+    rng = np.random.default_rng(n_mat)
+    n, n_pix = 20_000, 12
+    edges = np.logspace(np.log10(lo), np.log10(hi), n_mat + 1)
+    lens = crp.Lens(n_pix, np.zeros((n_mat, n_pix + 1), np.int64), np.zeros(0, np.int32), np.zeros(0, np.float32), edges)
+    p = I.make_particles(n, 3, species=(("H", .5), ("Fe", .5)))
+    R = 10.0 ** rng.uniform(np.log10(lo) - 1, np.log10(hi) + 1, n)
+    near = rng.integers(0, n, n // 2)
+    R[near] = rng.choice(edges, len(near)) * (1 + rng.choice([0.0, 1e-16, -1e-16, 1e-9, -1e-9, 1e-6, -1e-6], len(near)))
+    p.E[:] = R * p.Z
+    sim = crp.Simulation([crp.Field(np.zeros((4, 4, 4, 3), np.float32), I.MPC)], None, capacity=n)
+    sim.inject(p)
+    sim.propagate(1e-4, I.KPC, I.MPC, I.KPC)
+    assert sim.sync(60.0) == 0
+    s = sim.state()
+    st = O.OracleState(n)
+    O.inject(st, I.Particles(np.stack([s["x"], s["y"], s["z"]], 1), np.stack([s["ux"], s["uy"], s["uz"]], 1),
+                             s["E"], s["A"], s["Z"], s["uid"], s["grid_id"]), 1, None)
+    st.status[:n] = s["status"]
+    xo = O.lens_bin(st, 1, edges, 0.0)
+    assert xo.sum() > n // 2
+    assert np.array_equal(lens.bin(sim, 1, 0.0).cpu().numpy(), xo)
