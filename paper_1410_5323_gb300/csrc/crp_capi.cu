@@ -1496,12 +1496,17 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
     a.done_list = s->done_list;
     a.ctr = s->ctr;
     a.boundary = s->boundary == CRP_BOUNDARY_REFLECT ? 1 : 0;
+    double min_spacing = INFINITY;
+    for (const FieldDev& hf : s->host_fields) min_spacing = std::min(min_spacing, hf.spacing);
     for (int c = 0; c < 3; ++c) {
         a.box_lo[c] = s->box_origin[c];
         a.box_hi[c] = s->box_origin[c] + s->box_size[c];
         a.box_len[c] = s->box_size[c];
         a.box_inv[c] = s->boundary == CRP_BOUNDARY_REFLECT ? 1.0 / s->box_size[c] : 0.0;
-        a.box_lo_f[c] = (float)a.box_lo[c];
+        // FP32 images decide what is inside for certain. Where they or the margin (1e-6 of the box and more)
+        // would be subnormal they are NaN, which decides nothing.
+        const bool f32 = s->box_size[c] > 1e-30 && min_spacing > 1e-30;
+        a.box_lo_f[c] = f32 ? (float)a.box_lo[c] : NAN;
         a.box_hi_f[c] = (float)a.box_hi[c];
     }
     return CRP_OK;

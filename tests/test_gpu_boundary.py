@@ -164,3 +164,28 @@ def test_mixed_backtracking_returns_close_to_the_start():
     b = by_uid(bw.state())
     xb = np.stack([b["x"], b["y"], b["z"]], 1)
     assert np.median(np.linalg.norm(xb - p.x, axis=1)) < 1e-4 * d
+
+
+@pytest.mark.parametrize("size", [8.6e-45, 1.259e-44, 2e-43, 1e-40, 1e-30, 1e25, 1e28])
+def test_boxes_at_the_ends_of_the_float_range(size):
+    """Straight flight through 60 reflections in boxes whose FP32 images are subnormal, or whose sums
+    are near overflow: both forms end where the unfolded line, folded, ends."""
+    import paper_1410_5323_gb300 as crp
+
+    n = 500
+    p = I.make_particles(n, 7)
+    rng = np.random.default_rng(7)
+    lo, L = np.array([-0.3, 0.4, 0.0]) * size, np.array([1.0, 1.1, 0.9]) * size
+    p.x[:] = lo + rng.uniform(0.01, 0.99, (n, 3)) * L
+    d = 60 * size
+    t = (p.x + d * p.u - lo) / L % 2.0
+    want = lo + L * np.where(t > 1.0, 2.0 - t, t)
+    for form in (crp.FORM_FP64, crp.FORM_MIXED):
+        sim = crp.Simulation([crp.Field(np.zeros((4, 4, 4, 3), np.float32), size / 2)], None, capacity=n)
+        sim.set_boundary((lo, L))
+        sim.inject(p)
+        sim.propagate(1e-4, size / 1000, size / 7, d, form=form)
+        assert sim.sync(60.0) == 0
+        s = sim.state()
+        x = np.stack([s["x"], s["y"], s["z"]], 1)
+        assert np.max(np.abs(x - want)) < 1e-4 * size, form    # 420 steps, directions of FP32 pairs
