@@ -64,7 +64,8 @@ __device__ __forceinline__ void spectrum_consts(const crp_spectrum& sp, Spectrum
             K.lo = g != 0.0 ? lo : 0.0;
             K.hi = g != 0.0 ? hi : 0.0;
             K.lr = g != 0.0 ? 0.0 : crp_log(sp.e_max_ev / sp.e_min_ev);
-            K.W_f = (float)acc;
+            // below the normal FP32 numbers the sums' roundings are coarser than the margins: decided in FP64
+            K.W_f = acc > 1e-30 ? (float)acc : __int_as_float(0x7fc00000);
             K.ratio = (float)(hi / lo);
             K.inv_g = (float)(1.0 / g);
             K.lr2 = (float)(K.lr * 1.4426950408889634);

@@ -248,3 +248,23 @@ def test_healpix_pixels_on_both_sides_of_the_fp32_limit(oracle_lib, nside):
                         rng.standard_normal((200, 3)) * np.array([1.0, 1e-45, 1.0])])
     got = crp.healpix_ring(nside, torch.from_numpy(np.ascontiguousarray(u)).cuda()).cpu().numpy()
     assert np.array_equal(got, O.healpix_ring(nside, u))
+
+
+@pytest.mark.parametrize("scale,alpha,rcut,e_min,e_max", [
+    (3e-44, 1.8, RCUT, 1e18, 1e21), (3.3e-45, 1.0, RCUT, 1e18, 1e21), (1.36e-44, 1.0, RCUT, 1e18, 1e21),
+    (6.9e-46, 1.8, RCUT, 1e18, 1e21), (1e-300, 1.8, RCUT, 1e18, 1e21),
+    (1e300, 1.8, RCUT, 1e18, 1e21), (1.0, 1.0, 3e43, 1.0, 1e45), (1.0, 1.0, 1e300, 1e18, 1e21),
+    (1.0, 0.5, 1e-30, 1e-33, 1e-28), (1.0, 1.0, 1e41, 1e-300, 1e45)])
+def test_spectra_at_the_ends_of_the_float_range(scale, alpha, rcut, e_min, e_max):
+    """Abundances, cutoffs and ranges that FP32 holds as subnormals, as zero or not at all."""
+    import paper_1410_5323_gb300 as crp
+
+    n = 200_000
+    species = [(a, z, x * scale) for a, z, x in EQ1]
+    sim, _ = _sim(n, seed=31)
+    sim.sample_sources(crp.Spectrum.of(species, alpha, rcut, e_min, e_max), np.zeros((n, 3)))
+    s = sim.state()
+    A, Z, E, u, failed = O.source_sample(O.spectrum(species, alpha, rcut, e_min, e_max), 31, 0, n)
+    assert failed == np.sum(A == 0)
+    assert np.array_equal(s["A"], A) and np.array_equal(s["Z"], Z) and np.array_equal(s["E"], E)
+    assert np.array_equal(np.stack([s["ux"], s["uy"], s["uz"]], 1), u)
