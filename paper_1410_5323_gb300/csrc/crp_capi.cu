@@ -531,6 +531,18 @@ long long list_length(const crp_sim* s, long long capacity) {
     return capacity + std::min(capacity, (long long)std::max(1, s->sms) * kThreadsPerSm);
 }
 
+// Steps per slot for particles handed between launches (FP64 form), or NULL where there is no room for
+// them: particles then stay in the launch that took them. Called where a simulation allocates, never in a
+// call that finds its copies made (which may be under stream capture).
+int32_t* alloc_taken(long long capacity) {
+    int32_t* p = nullptr;
+    if (dev_malloc(&p, sizeof(int32_t) * capacity) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return p;
+}
+
 int sync_stream(crp_sim* s) {
     cudaError_t e = cudaStreamSynchronize(s->last);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
@@ -780,7 +792,6 @@ int crp_sim_create(const crp_field* const* fields, int32_t n_fields, const crp_t
     if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->lists[0], sizeof(int32_t) * list_length(s, capacity));
     if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->lists[1], sizeof(int32_t) * list_length(s, capacity));
     if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->done_list, sizeof(int32_t) * capacity);
-    if (rc == CRP_OK && e == cudaSuccess && layout == LAYOUT_F64X4) e = dev_malloc(&s->taken, sizeof(int32_t) * capacity);
     if (rc == CRP_OK && e == cudaSuccess) e = dev_malloc(&s->ctr, sizeof(Counters));
     if (rc == CRP_OK && e == cudaSuccess) e = cudaMemset(s->ctr, 0, sizeof(Counters));
     const size_t sort_bytes = 2 * (size_t)kBuckets * n_fields * sizeof(unsigned);
@@ -790,6 +801,7 @@ int crp_sim_create(const crp_field* const* fields, int32_t n_fields, const crp_t
         crp_sim_destroy(s);
         return rc != CRP_OK ? rc : cuda_fail(e, "crp_sim_create allocations");
     }
+    if (layout == LAYOUT_F64X4) s->taken = alloc_taken(capacity);
     *out = s;
     return CRP_OK;
 }
@@ -863,7 +875,7 @@ int crp_sim_reserve(crp_sim* s, int64_t capacity) {
     cudaError_t e = dev_malloc(&l0, sizeof(int32_t) * list_length(s, capacity));
     if (e == cudaSuccess) e = dev_malloc(&l1, sizeof(int32_t) * list_length(s, capacity));
     if (e == cudaSuccess) e = dev_malloc(&dl, sizeof(int32_t) * capacity);
-    if (e == cudaSuccess && s->taken) e = dev_malloc(&tk, sizeof(int32_t) * capacity);
+    if (e == cudaSuccess && s->taken) tk = alloc_taken(capacity);
     if (e == cudaSuccess) e = cudaMemset(&s->ctr->tidy, 0, sizeof(int));   // new lists
     for (int c = 0; c < CRP_N_COLS && e == cudaSuccess; ++c)
         e = cudaMemcpy(*col_ptr(ns, c), *col_ptr(s->st, c), (size_t)h.n_used * kCols[c].size,
@@ -1305,8 +1317,7 @@ int field_fp64_desc(crp_field* f, FieldDev& out) {
 }
 
 // Build (once per field) the FP64 copies and this simulation's descriptor array for them.
-int ensure_fp64_fields(crp_sim* s) {
-    if (s->d_fields64) return CRP_OK;
+int make_fp64_fields(crp_sim* s) {
     int rc = sync_stream(s);
     if (rc) return rc;
     std::vector<FieldDev> d64;
@@ -1328,6 +1339,23 @@ int ensure_fp64_fields(crp_sim* s) {
     if (e != cudaSuccess) { cudaFree(d); return cuda_fail(e, "cudaMemcpy(fields64)"); }
     s->d_fields64 = (FieldDev*)d;
     return CRP_OK;
+}
+
+int ensure_fp64_fields(crp_sim* s) {
+    if (s->d_fields64) return CRP_OK;
+    s->taken = alloc_taken(s->capacity);
+    int rc = make_fp64_fields(s);
+    if (rc == CRP_ERR_OOM && s->taken) {      // the copies come first
+        cudaGetLastError();
+        cudaFree(s->taken);
+        s->taken = nullptr;
+        rc = make_fp64_fields(s);
+    }
+    if (rc && s->taken) {
+        cudaFree(s->taken);
+        s->taken = nullptr;
+    }
+    return rc;
 }
 
 // Cell-major copies (precision form): bytes they need beyond what is already built.
@@ -1398,8 +1426,6 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
         if (rc) return rc;
         fields = s->d_fields64;
         layout = LAYOUT_F64X4;
-        // without room for it particles stay in the launch that took them
-        if (!s->taken && dev_malloc(&s->taken, sizeof(int32_t) * s->capacity) != cudaSuccess) cudaGetLastError();
     }
     if (prm->grid_layout != CRP_GRID_AUTO && prm->grid_layout != CRP_GRID_NODES &&
         prm->grid_layout != CRP_GRID_CELLS)

@@ -138,3 +138,34 @@ def test_calls_with_and_without_pickup_on_one_simulation():
             states.append(by_uid(sim.state()))
         for s in states[1:]:
             assert_bit_identical(states[0], s)
+
+
+def test_no_room_for_the_hand_over_and_under_capture(oracle_lib):
+    """The first allocation of the first FP64 call fails (the steps of particles handed on): that call
+    and a captured one, which must not allocate, finish in the launches that took the particles."""
+    import torch
+
+    import paper_1410_5323_gb300 as crp
+
+    n = 60_000
+    p = I.make_particles(n, 3, species=MIX, energy=("power", 3e18, 10 ** 20.5, 2.0))
+    t = I.constant_rate_tables(0.0, 1 / (3 * I.MPC))
+    args = (1e-4, I.KPC, I.MPC, 2 * I.MPC)
+    sim = crp.Simulation([crp.Field(_grid(16, 6), 0.25 * I.MPC)], crp.Tables(t), seed=9, capacity=6 * n)
+    sim.inject(p)
+    try:
+        crp.debug_fail_allocations(1)
+        sim.propagate(*args, max_steps=4)
+    finally:
+        crp.debug_fail_allocations(0)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        sim.propagate(*args, max_steps=4)
+    for _ in range(5):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert sim.sync(60.0) == 0
+    st, rc = run_oracle([_grid(16, 6)], p, t, *args, seed=9, capacity=6 * n, max_steps=4, calls=6)
+    assert rc == 0
+    assert_bit_identical(sim.state(), st.snapshot())
