@@ -2034,13 +2034,14 @@ int crp_adjoint_create(const crp_field* field, int64_t n, int32_t n_steps, int32
     int rc = field_fp64_desc(a->field, F);
     if (rc) { adj_free(a); delete a; return rc; }
     // stage records of all steps (kAdjRecordBytes per step and particle) when they fit in half
-    // of the free memory and the grid's node indices fit in int32: every segment's records are
-    // then formed in parallel and the serial reverse sweep only applies them
+    // of the free memory and the grid's node indices fit in int32: every step's records are
+    // then formed in parallel and the serial reverse sweep only applies them. The states they are formed
+    // from (a twenty-seventh of that) come out of the other half.
     size_t free_b = 0, total_b = 0;
     const size_t st_bytes = kAdjRecordBytes * (size_t)n_steps * (size_t)n;
     const size_t y_bytes = 6 * sizeof(double) * (size_t)n_steps * (size_t)n;
     const long long nodes = (long long)F.nx * F.ny * F.nz;
-    if (nodes < (1ll << 31) && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && st_bytes + y_bytes <= free_b / 2) {
+    if (nodes < (1ll << 31) && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && st_bytes <= free_b / 2) {
         if (dev_malloc(&a->stages, st_bytes) != cudaSuccess) {
             a->stages = nullptr;
             cudaGetLastError();
