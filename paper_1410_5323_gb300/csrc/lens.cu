@@ -179,9 +179,11 @@ __global__ void __launch_bounds__(64) k_lens_apply_maps(int n_pix, int n_maps, i
                 A = B;
                 k += kPipe;
             }
+            if (k < len) {      // a predicated-off DFMA takes its turn of the FP64 unit all the same
 #pragma unroll
-            for (int t = 0; t < kPipe; ++t)
-                if (k + t < len) acc = __fma_rn(widen<PLAIN>(A.v[t]), A.x[t], acc);
+                for (int t = 0; t < kPipe; ++t)
+                    if (k + t < len) acc = __fma_rn(widen<PLAIN>(A.v[t]), A.x[t], acc);
+            }
         }
         y[p * n_maps + b] = acc;
     }
