@@ -201,3 +201,18 @@ def test_rigidity_bins_at_the_ends_of_the_float_range(oracle_lib, lo, hi, n_mat)
     xo = O.lens_bin(st, 1, edges, 0.0)
     assert xo.sum() > n // 2
     assert np.array_equal(lens.bin(sim, 1, 0.0).cpu().numpy(), xo)
+
+
+@pytest.mark.parametrize("n_maps", [64, 96, 97])
+def test_whole_groups_of_maps_bit_identical(oracle_lib, n_maps):
+    """Two and three groups of 32 maps in one launch, and one map after them."""
+    import paper_1410_5323_gb300 as crp
+
+    rng = np.random.default_rng(n_maps)
+    n_pix = 77
+    counts = rng.integers(0, 13, n_pix)
+    rp = np.concatenate([[0], np.cumsum(counts)]).astype(np.int64)[None]
+    col = rng.integers(0, n_pix, int(rp[0, -1])).astype(np.int32)
+    val = rng.standard_normal(len(col)).astype(np.float32)
+    x = rng.standard_normal((1, n_pix, n_maps))
+    assert np.array_equal(_gpu(crp.Lens(n_pix, rp, col, val), x), O.lens_apply(n_pix, rp, col, val, x))
