@@ -110,9 +110,10 @@ __device__ __forceinline__ bool sure_floor(float v, float eps, int& i) {
 // ordinary numbers. Bounds: z/r and phi / (pi/2) are off by less than 1e-6 (inputs 2^-23 relative,
 // atan2f 3 ulp of pi, rsqrtf 2 ulp); twice that is used, and the sums' own roundings.
 __device__ __forceinline__ int healpix_ring_f32(int ns, double dx, double dy, double dz) {
+    if (ns > kFastNside) return -2;
     const float x = head_f32(dx), y = head_f32(dy), z = head_f32(dz);
     const float r2 = fmaf(x, x, fmaf(y, y, z * z));
-    if (!(r2 > 1e-20f && r2 < 1e20f) || ns > kFastNside) return -2;
+    if (!(r2 > 1e-20f && r2 < 1e20f)) return -2;
     const float zz = z * rsqrtf(r2);
     float t = atan2f(y, x) * 0.63661977f;
     if (t < 0.0f) t += 4.0f;
