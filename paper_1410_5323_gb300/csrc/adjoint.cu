@@ -676,7 +676,7 @@ int adj_record(const FieldDev& F, const double* y0, const double* kappa, double 
     const long long warps = (n + per_warp - 1) / per_warp;
     // Up to four warps per SM: blocks of four, with shared memory that a second one finds no room for.
     // More: one-warp blocks, which are dealt out evenly (7000 chains of 200 steps in blocks of four:
-    // 4.42 ms, since some SMs then had eight warps and others four; 3.61 ms in blocks of one).
+    // 4.42 ms, since some SMs then had eight warps and others four; 3.39 ms in blocks of one).
     const bool one_layer = warps <= 4 * sms;
     const int shm = one_layer ? kOnePerSmBytes : 0, block = one_layer ? 128 : 32;
     if (shm) {
