@@ -130,8 +130,11 @@ __device__ __forceinline__ void floor_weights(double r, long long& i, double& w0
 // One axis of the periodic lookup: r = x (1/spacing) - o (1/spacing) with one rounding (oi is
 // the product o (1/spacing), rounded once), i0 = floor(r) mod n, weights (1 - f, f). P2: the
 // caller guarantees n is a power of two, and the 64-bit modulo's code (inlined at every
-// lookup, never run for such grids) is left out of the kernel.
-template <bool P2 = false>
+// lookup, never run for such grids) is left out of the kernel. Rem32: indices that fit take the 32-bit
+// remainder, a third of the 64-bit one (300 000 protons on 100^3 over 20 Mpc 74.2 -> 67.9 ms). Not with a
+// modulation, whose six more axes make the branches' code outweigh it (the same on 100^3 modulated by
+// 64^3 116.6 ms with the 64-bit remainder alone, 127.6 with both; 10^6 Sec. 4 sources 5.36 and 5.50 s).
+template <bool P2 = false, bool Rem32 = true>
 __device__ __forceinline__ void axis(double x, double oi, double inv, int n, int pow2,
                                      long long& i0, long long& i1, double& w0, double& w1) {
     const double r = __fma_rn(x, inv, -oi);
@@ -143,7 +146,7 @@ __device__ __forceinline__ void axis(double x, double oi, double inv, int n, int
     long long a;
     if (P2 || pow2) {
         a = i & (long long)(n - 1);
-    } else if (i == (long long)(int)i) {   // the 32-bit remainder is a third of the 64-bit one
+    } else if (Rem32 && i == (long long)(int)i) {
         a = (int)i % n;
         if (a < 0) a += n;
     } else {
@@ -160,9 +163,9 @@ __device__ __forceinline__ void axis(double x, double oi, double inv, int n, int
 __device__ __forceinline__ double modulation(const FieldDev& F, double x, double y, double z) {
     long long ix0, ix1, iy0, iy1, iz0, iz1;
     double wx0, wx1, wy0, wy1, wz0, wz1;
-    axis(x, F.moix, F.m_inv_spacing, F.mnx, F.mpow2, ix0, ix1, wx0, wx1);
-    axis(y, F.moiy, F.m_inv_spacing, F.mny, F.mpow2, iy0, iy1, wy0, wy1);
-    axis(z, F.moiz, F.m_inv_spacing, F.mnz, F.mpow2, iz0, iz1, wz0, wz1);
+    axis<false, false>(x, F.moix, F.m_inv_spacing, F.mnx, F.mpow2, ix0, ix1, wx0, wx1);
+    axis<false, false>(y, F.moiy, F.m_inv_spacing, F.mny, F.mpow2, iy0, iy1, wy0, wy1);
+    axis<false, false>(z, F.moiz, F.m_inv_spacing, F.mnz, F.mpow2, iz0, iz1, wz0, wz1);
     const long long ny = F.mny, nz = F.mnz;
     const float* M = F.mod;
     const long long r00 = (ix0 * ny + iy0) * nz, r01 = (ix0 * ny + iy1) * nz;
@@ -193,9 +196,9 @@ __device__ __forceinline__ V3 field_b(const FieldDev& F, double x, double y, dou
                                       unsigned long long* hh = nullptr) {
     long long ix0, ix1, iy0, iy1, iz0, iz1;
     double wx0, wx1, wy0, wy1, wz0, wz1;
-    axis<P2>(x, F.oix, F.inv_spacing, F.nx, F.pow2, ix0, ix1, wx0, wx1);
-    axis<P2>(y, F.oiy, F.inv_spacing, F.ny, F.pow2, iy0, iy1, wy0, wy1);
-    axis<P2>(z, F.oiz, F.inv_spacing, F.nz, F.pow2, iz0, iz1, wz0, wz1);
+    axis<P2, !M>(x, F.oix, F.inv_spacing, F.nx, F.pow2, ix0, ix1, wx0, wx1);
+    axis<P2, !M>(y, F.oiy, F.inv_spacing, F.ny, F.pow2, iy0, iy1, wy0, wy1);
+    axis<P2, !M>(z, F.oiz, F.inv_spacing, F.nz, F.pow2, iz0, iz1, wz0, wz1);
     const long long ny = F.ny, nz = F.nz;
     if constexpr (H) *hh = *hh * 0x9E3779B97F4A7C15ull + (unsigned long long)((ix0 * ny + iy0) * nz + iz0) + 1ull;
     const long long r00 = (ix0 * ny + iy0) * nz, r01 = (ix0 * ny + iy1) * nz;
