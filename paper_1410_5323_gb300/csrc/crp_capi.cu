@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <chrono>
+#include <climits>
 #include <cstdint>
 #include <mutex>
 #include <cmath>
@@ -347,17 +348,17 @@ __global__ void k_build_worklist(const int32_t* __restrict__ status, int32_t* __
 }
 
 // After a propagate launch over list C->cur: fix the slot count, reset the pop head and the list
-// that the next launch pushes into, and make the other list the next one. A one-lane launch that
-// left its list alone (at most min_work entries) changes nothing. One block; in calls that take
+// that the next launch pushes into, and make the other list the next one. A launch that left its list
+// alone (not more than lo or more than hi entries) changes nothing. One block; in calls that take
 // secondaries up (l0 not NULL) it puts -1 back into the list, whose entries would otherwise pass for
 // published ones when a launch pushes into it. (Left to whoever takes an entry, that store slowed the
 // launch: 10^6 sources of a sky map 1.8 -> 2.5 ms, 10^6 nuclei 68 -> 73 ms.)
-__global__ void k_swap(Counters* C, long long capacity, long long min_work, int32_t* l0, int32_t* l1) {
+__global__ void k_swap(Counters* C, long long capacity, long long lo, long long hi, int32_t* l0, int32_t* l1) {
     CRP_COUNT_RUN();
     const int from = C->cur;
-    const long long n = (long long)C->count[from];
+    const long long n = (long long)C->count[from], work = n - (long long)C->head0;
     if (l0 && threadIdx.x == 0) C->tidy = 1;
-    if (n - (long long)C->head0 <= min_work) return;
+    if (work <= lo || work > hi) return;
     if (l0) {
         int32_t* l = from ? l1 : l0;
         for (long long i = threadIdx.x; i < n; i += blockDim.x) l[i] = -1;
@@ -446,15 +447,25 @@ void** col_ptr(SimState& S, int c) {
 
 // ---- handles ------------------------------------------------------------------------------
 namespace {
+// One propagate launch of a call: its shape, and the lists that it takes (PropArgs::min_work, max_work).
+// FULL: the one-lane kernel of the form, as many blocks as run at once. TEAM: three lanes per particle, as
+// many blocks as run at once. LAYER: one block per SM, of the three-lane kernel (FP64 form) or with the
+// particles dealt out evenly (precision form).
+enum StepKind : int32_t { STEP_FULL, STEP_TEAM, STEP_LAYER };
+struct Step {
+    int32_t kind, pickup;
+    long long lo, hi;
+    long long drain_at;              // PropArgs::drain_at, -1: particles stay in the launch
+};
+
 // One validated propagate call: kernel arguments and launch shape.
 struct Plan {
     PropArgs a{};
     int grid = 0, block = 0, order = 0, mixed = 0, n_buckets = 0, layout = 0, mod = 0;
     int p2 = 0;   // every field's vector grid has power-of-two sizes
-    int team_grid = 0, team_block = 0;   // three-lane kernel: blocks (0: not launched), threads per block
-    int team_launches = 0;
-    int lane_launches = 2;               // launches of the one-lane kernel before those
-    int spread_launches = 0;             // launches of the precision form with one block per SM after those
+    int team_grid = 0;                   // blocks of STEP_TEAM
+    int n_steps = 0;
+    Step steps[7] = {};
 };
 
 }  // namespace
@@ -1468,27 +1479,56 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
     if (team) bps = std::min(bps, kThreadsPerSm / block);   // no more than run at once: list_length
     P.grid = sms * bps;
     const long long lanes = (long long)P.grid * block;
-    // Without tables there are no secondaries and one launch does; with them the second takes those
-    // that the first left (all, if they wait for it).
-    P.team_grid = P.team_block = P.team_launches = P.spread_launches = 0;
-    P.lane_launches = mixed && !s->tables ? 1 : 2;
-    // Precision form: lists that fit one block per SM go to launches of that shape, which deal the
-    // particles out evenly (1024 protons over 100 Mpc: 764 -> 568 us; 19 000 over 50 Mpc: 1076 -> 961 us).
-    const long long one_layer = (long long)sms * block;
-    if (mixed && prm->blocks_per_sm <= 0) {
-        P.spread_launches = s->tables ? 2 : 1;
-        P.lane_launches = s->capacity <= one_layer ? 0 : (s->tables && pickup == CRP_PICKUP_OFF ? 2 : 1);
-    }
+    // The launches of the call, by the sizes of the lists they take. Without tables there are no secondaries.
+    // With them the secondaries of a list are the next launch's list, of any size, so every shape comes again
+    // after the first that can release many: 19 000 iron nuclei end as 174 000 or 760 000 nucleons, and with
+    // those in one block per SM the calls took 5.6 and 2.7 ms, with all lanes 3.5 and 1.5 (precision form; FP64
+    // form 12.4 and 17.9, 8.4 and 10.1 ms). A launch whose list is of another size ends at once (6 us with its
+    // bookkeeping).
+    constexpr long long kAny = LLONG_MAX;
+    P.team_grid = P.n_steps = 0;
+    auto step = [&](StepKind kind, long long lo, long long hi, long long drain_at = -1) {
+        P.steps[P.n_steps++] = Step{kind, take_up, lo, hi, drain_at};
+    };
+    const long long cap = s->capacity;
     if (team) {
         int occ = prm->blocks_per_sm;
         if (occ <= 0 && (propagate_team_occupancy(s->mod, p2, block, &occ) != 0 || occ < 1)) occ = 1;
         P.team_grid = sms * std::min(occ, kThreadsPerSm / block);
-        P.team_block = block;
-        P.lane_launches = s->capacity <= lanes ? 0 : (s->tables && pickup == CRP_PICKUP_OFF ? 2 : 1);
-        // what one block per SM takes up needs no launch that drains
-        a.drain_at = (long long)sms * (block / 32) * kTeamsPerWarp;
-        P.team_launches = s->capacity <= a.drain_at || !s->tables ? 2 : 3;
+        const long long layer = (long long)sms * (block / 32) * kTeamsPerWarp;   // particles of STEP_LAYER
+        // Handed on by STEP_FULL once half of the lanes hold a particle: full lanes are worth more than teams
+        // (10^6 nuclei over 500 Mpc: 7473 ms handing on as soon as the list has run out, 7173 at 6/8 or
+        // less; 10^6 in a modulated field 5598 at 6/8, 5506 at 4/8, 5513 never; 60 000 over 100 Mpc: 285
+        // without teams, 141 at once, 138 at 6/8, 140 at 4/8, 147 at 2/8), by STEP_TEAM once one block per SM
+        // holds them.
+        const long long to_team = s->taken ? lanes / 2 : -1, to_layer = s->taken ? layer : -1;
+        if (s->tables && cap > layer) {
+            step(STEP_LAYER, -1, layer);
+            step(STEP_TEAM, layer, cap > lanes ? lanes : kAny, to_layer);
+        }
+        if (cap > lanes) {
+            step(STEP_FULL, lanes, kAny, to_team);
+            if (s->tables) step(STEP_FULL, lanes, kAny, to_team);
+        }
+        if (cap > layer && (cap > lanes || !s->tables)) step(STEP_TEAM, layer, kAny, to_layer);
+        if (cap <= layer || s->tables) step(STEP_LAYER, -1, kAny);
+        step(STEP_LAYER, -1, kAny);
+    } else if (mixed && prm->blocks_per_sm <= 0) {
+        // lists that fit one block per SM go to launches of that shape, which deal the particles out evenly
+        // (1024 protons over 100 Mpc: 764 -> 568 us; 19 000 over 50 Mpc: 1076 -> 961 us)
+        const long long layer = (long long)sms * block;
+        if (s->tables) step(STEP_LAYER, -1, cap > layer ? layer : kAny);
+        if (cap > layer) {
+            step(STEP_FULL, layer, kAny);
+            if (s->tables) step(STEP_FULL, layer, kAny);
+        }
+        step(STEP_LAYER, -1, kAny);
+        for (int k = s->tables && cap > layer ? 2 : 1; k < P.n_steps; ++k) P.steps[k].pickup = 0;
+    } else {
+        step(STEP_FULL, -1, kAny);
+        if (!mixed || s->tables) step(STEP_FULL, -1, kAny);
     }
+    if (s->tables) P.steps[P.n_steps - 1].pickup = 0;      // nucleons, which release nothing
     P.block = block;
     P.order = order;
     P.mixed = mixed ? 1 : 0;
@@ -1513,8 +1553,7 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
     a.cadence = prm->cadence > 0 ? prm->cadence : (!mixed ? 1 : (take_up ? 2 : 8));
     a.pickup = take_up;
     a.spread = 0;
-    a.drain = team && s->taken ? 1 : 0;
-    a.min_work = team ? lanes : (P.spread_launches ? one_layer : -1);
+    a.drain = 0;
     a.taken = team ? s->taken : nullptr;
     a.back = team ? 1 : 0;
     a.lists[0] = s->lists[0];
@@ -1566,45 +1605,25 @@ int enqueue(crp_sim* s, const Plan& P, cudaStream_t st) {
                                               grid_major, offs, s->lists[0], s->ctr);
     }
     CRP_CUDA(cudaGetLastError());
-    // generation 1: the work list (and, with pickup, secondaries it pushes once the list
-    // runs dry); generation 2: the secondaries left. Nucleon secondaries never split, so two
-    // launches finish the call. With the three-lane kernel a one-lane launch hands its active
-    // particles on when its list has run out and its lanes are emptying, to the next list with the
-    // secondaries, and the three-lane launches finish them.
-    for (int gen = 0; gen < P.lane_launches; ++gen) {
+    // Each launch takes the list that the one before it left: the work list first, then the secondaries and, in
+    // the FP64 form, the particles handed on. Nucleon secondaries never split.
+    for (int k = 0; k < P.n_steps; ++k) {
+        const Step& step = P.steps[k];
         PropArgs l = a;
-        // Handed on once half of the lanes hold a particle: full lanes are worth more than teams
-        // (10^6 nuclei over 500 Mpc: 7473 ms handing on as soon as the list has run out, 7173 at 6/8 or
-        // less; 10^6 in a modulated field 5598 at 6/8, 5506 at 4/8, 5513 never; 60 000 over 100 Mpc: 285
-        // without teams, 141 at once, 138 at 6/8, 140 at 4/8, 147 at 2/8).
-        if (a.drain) l.drain_at = a.min_work / 2;
-        int e = P.mixed ? launch_propagate_mixed(l, P.layout, P.mod, P.p2, P.grid, P.block, st)
-                        : launch_propagate_fp64(l, P.layout, P.mod, P.p2, P.grid, P.block, st);
+        l.pickup = step.pickup;
+        l.min_work = step.lo;
+        l.max_work = step.hi;
+        l.drain_at = step.drain_at;
+        l.drain = step.drain_at >= 0 ? 1 : 0;
+        l.spread = P.mixed && step.kind == STEP_LAYER ? 1 : 0;
+        const bool layer = step.kind == STEP_LAYER;
+        const int grid = layer ? std::max(1, s->sms) : (step.kind == STEP_TEAM ? P.team_grid : P.grid);
+        int e;
+        if (P.mixed) e = launch_propagate_mixed(l, P.layout, P.mod, P.p2, grid, P.block, st);
+        else if (step.kind == STEP_FULL) e = launch_propagate_fp64(l, P.layout, P.mod, P.p2, grid, P.block, st);
+        else e = launch_propagate_team(l, P.mod, P.p2, grid, P.block, layer ? 1 : 0, st);
         if (e) return cuda_fail((cudaError_t)e, "propagate kernel launch");
-        k_swap<<<1, tidy ? 1024 : 1, 0, st>>>(s->ctr, s->capacity, a.min_work, l0, s->lists[1]);
-        CRP_CUDA(cudaGetLastError());
-    }
-    for (int gen = 0; gen < P.spread_launches; ++gen) {
-        PropArgs t = a;
-        t.spread = 1;
-        t.min_work = -1;
-        if (gen > 0) t.pickup = 0;      // nucleons: they release nothing
-        int e = launch_propagate_mixed(t, P.layout, P.mod, P.p2, std::max(1, s->sms), P.block, st);
-        if (e) return cuda_fail((cudaError_t)e, "propagate kernel launch");
-        k_swap<<<1, tidy ? 1024 : 1, 0, st>>>(s->ctr, s->capacity, -1, l0, s->lists[1]);
-        CRP_CUDA(cudaGetLastError());
-    }
-    for (int gen = 0; gen < P.team_launches; ++gen) {
-        // one that drains if the particles may not fit one block per SM, one for what is left, and one
-        // for the secondaries that this released late (nucleons, which release nothing)
-        PropArgs t = a;
-        t.drain = a.drain && gen == 0 && s->capacity > a.drain_at ? 1 : 0;
-        t.min_work = t.drain ? a.drain_at : -1;
-        if (gen == P.team_launches - 1) t.pickup = 0;
-        int e = launch_propagate_team(t, P.mod, P.p2, t.drain ? P.team_grid : std::max(1, s->sms), P.team_block,
-                                      t.drain ? 0 : 1, st);
-        if (e) return cuda_fail((cudaError_t)e, "propagate kernel launch");
-        k_swap<<<1, tidy ? 1024 : 1, 0, st>>>(s->ctr, s->capacity, t.min_work, l0, s->lists[1]);
+        k_swap<<<1, tidy ? 1024 : 1, 0, st>>>(s->ctr, s->capacity, step.lo, step.hi, l0, s->lists[1]);
         CRP_CUDA(cudaGetLastError());
     }
     return CRP_OK;
@@ -1630,9 +1649,8 @@ __global__ void k_loop_cond(Counters* C, cudaGraphConditionalHandle h, long long
 bool same_plan(const Plan& x, const Plan& y) {
     return std::memcmp(&x.a, &y.a, sizeof(PropArgs)) == 0 && x.grid == y.grid &&
            x.block == y.block && x.order == y.order && x.mixed == y.mixed && x.n_buckets == y.n_buckets &&
-           x.p2 == y.p2 && x.team_grid == y.team_grid && x.team_block == y.team_block &&
-           x.team_launches == y.team_launches &&
-           x.lane_launches == y.lane_launches && x.spread_launches == y.spread_launches && x.layout == y.layout && x.mod == y.mod;
+           x.p2 == y.p2 && x.team_grid == y.team_grid && x.n_steps == y.n_steps &&
+           std::memcmp(x.steps, y.steps, sizeof(Step) * x.n_steps) == 0 && x.layout == y.layout && x.mod == y.mod;
 }
 
 }  // namespace
@@ -1951,10 +1969,11 @@ extern "C" int crp_propagate_noalloc(const void* grid, int32_t nx, int32_t ny, i
     a.done_list = done;
     a.ctr = ctr;
     a.min_work = -1;
+    a.max_work = LLONG_MAX;
     for (int gen = 0; gen < 2; ++gen) {
         int e = launch_propagate_fp64(a, LAYOUT_F32X4, 0, f.pow2, sms * occ, block, st);
         if (e) return cuda_fail((cudaError_t)e, "propagate kernel launch");
-        k_swap<<<1, 1, 0, st>>>(ctr, n, -1, nullptr, nullptr);
+        k_swap<<<1, 1, 0, st>>>(ctr, n, -1, LLONG_MAX, nullptr, nullptr);
         CRP_CUDA(cudaGetLastError());
     }
     CRP_CUDA(cudaStreamSynchronize(st));

@@ -111,7 +111,8 @@ struct PropArgs {
                                      // active particles on to the next launch
     int32_t back;                    // lists that a launch of this call filled are taken from their end
     long long drain_at;
-    long long min_work;              // a launch leaves lists of at most this many entries to the next one
+    long long min_work, max_work;    // a launch takes lists of more than min_work and at most max_work entries
+                                     // and leaves others to the next one
     int32_t* taken;                  // per slot: accepted steps of this call so far (drained particles); may be NULL
     int32_t* lists[2];               // list Counters::cur is processed, secondaries are pushed to the other
     int32_t* done_list;

@@ -60,6 +60,10 @@ struct WorkList {
     int L;
     bool back;
     unsigned long long n_work, head0;
+    __device__ __forceinline__ bool fits(const PropArgs& a) const {
+        const long long n = (long long)(n_work - head0);
+        return n > a.min_work && n <= a.max_work;
+    }
 };
 __device__ __forceinline__ WorkList work_list(const PropArgs& a) {
     const Counters* C = a.ctr;

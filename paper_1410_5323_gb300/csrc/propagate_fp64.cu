@@ -51,7 +51,7 @@ __global__ void CRP_FP64_BOUNDS k_propagate_fp64(const PropArgs a) {
     Counters* C = a.ctr;
     const WorkList work = work_list(a);
     const int pushes = 1 - work.L;
-    if ((long long)(work.n_work - work.head0) <= a.min_work) return;
+    if (!work.fits(a)) return;
     const double INF = __longlong_as_double(0x7ff0000000000000LL);
     const SimState& S = a.st;
 

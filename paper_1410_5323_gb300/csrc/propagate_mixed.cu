@@ -350,7 +350,7 @@ __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* s
     Counters* C = a.ctr;
     const WorkList work = work_list(a);
     const int pushes = 1 - work.L;
-    if ((long long)(work.n_work - work.head0) <= a.min_work) return;
+    if (!work.fits(a)) return;
     const float INF = __int_as_float(0x7f800000);
     const SimState& S = a.st;
     // a batch that can't fill one block per SM: evenly over the warps, since the lanes of a warp wait

@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(256, M ? 1 : 2) k_propagate_fp64_team(const Pr
     Counters* C = a.ctr;
     const WorkList work = work_list(a);
     const int pushes = 1 - work.L;
-    if ((long long)(work.n_work - work.head0) <= a.min_work) return;
+    if (!work.fits(a)) return;
     // fewer particles than teams: evenly over the warps
     const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
     const int quota = (int)min((unsigned long long)kTeams, (work.n_work - work.head0 + warps - 1) / warps);

@@ -169,3 +169,78 @@ def test_no_room_for_the_hand_over_and_under_capture(oracle_lib):
     st, rc = run_oracle([_grid(16, 6)], p, t, *args, seed=9, capacity=6 * n, max_steps=4, calls=6)
     assert rc == 0
     assert_bit_identical(sim.state(), st.snapshot())
+
+
+def _run(grid, p, t, args, *, seed, capacity, calls=1, loop=False, **kw):
+    import paper_1410_5323_gb300 as crp
+
+    sim = crp.Simulation([crp.Field(grid, 0.25 * I.MPC)], crp.Tables(t), seed=seed, capacity=capacity)
+    sim.inject(p)
+    for _ in range(calls):
+        (sim.propagate_loop if loop else sim.propagate)(*args, **kw)
+    assert sim.sync(60.0) == 0
+    return sim.state()
+
+
+@pytest.mark.parametrize("n", [200, 3000, 20_000])
+def test_iron_releases_lists_of_every_size(oracle_lib, n):
+    """18 nucleons for each iron nucleus: the secondaries' list takes another launch shape than the
+    nuclei's, and is above and below what idle lanes take up, in every pick-up mode."""
+    import paper_1410_5323_gb300 as crp
+
+    p = I.make_particles(n, 15, species=(("Fe", 1.0),), energy=("power", 10 ** 19.5, 10 ** 20.5, 2.0))
+    g, t, args = _grid(16, 10), I.constant_rate_tables(0.0, 1 / (0.1 * I.MPC)), (1e-4, I.KPC, I.MPC, 2 * I.MPC)
+    kw = dict(seed=8, capacity=40 * n)
+    st, rc = run_oracle([g], p, t, *args, **kw)
+    assert rc == 0 and len(st.snapshot()["uid"]) > 12 * n
+    plain = _run(g, p, t, args, form=crp.FORM_MIXED, pickup=1, blocks_per_sm=2, **kw)
+    for mode in (0, 1, 2):
+        assert_bit_identical(_run(g, p, t, args, form=crp.FORM_FP64, pickup=mode, **kw), st.snapshot())
+        assert_bit_identical(_run(g, p, t, args, form=crp.FORM_MIXED, pickup=mode, **kw), plain)
+
+
+@pytest.mark.parametrize("pickup,max_steps,calls", [(0, 0, 1), (0, 4, 6), (2, 0, 1)])
+def test_lists_above_twelve_fills_of_the_lanes(oracle_lib, pickup, max_steps, calls):
+    """4864 lanes for 60 000 nuclei and their secondaries, which wait for the list's end."""
+    p = I.make_particles(60_000, 3, species=MIX, energy=("power", 3e18, 10 ** 20.5, 2.0))
+    g, t, args = _grid(16, 6), I.constant_rate_tables(0.0, 1 / (3 * I.MPC)), (1e-4, I.KPC, I.MPC, 2 * I.MPC)
+    kw = dict(seed=9, capacity=6 * 60_000, max_steps=max_steps, calls=calls)
+    st, rc = run_oracle([g], p, t, *args, **kw)
+    assert rc == 0
+    assert_bit_identical(_run(g, p, t, args, pickup=pickup, block_size=32, blocks_per_sm=1, **kw), st.snapshot())
+
+
+@pytest.mark.parametrize("form", [0, 1])
+def test_graph_loop_through_every_launch(oracle_lib, form):
+    """Slices whose list begins above the lanes and ends below one block per SM, the lists' state kept on
+    the device between them: the FP64 form against the oracle, the precision form against calls."""
+    n = 90_000
+    p = I.make_particles(n, 17, species=MIX, energy=("power", 3e18, 10 ** 20.5, 2.0))
+    g, t, args = _grid(16, 6), I.constant_rate_tables(0.0, 1 / (3 * I.MPC)), (1e-4, I.KPC, I.MPC, 2 * I.MPC)
+    kw = dict(seed=9, capacity=6 * n)
+    got = _run(g, p, t, args, form=form, max_steps=4, loop=True, **kw)
+    if form == 0:
+        st, rc = run_oracle([g], p, t, *args, **kw)
+        assert rc == 0
+        assert_bit_identical(got, st.snapshot())
+    else:
+        assert_bit_identical(got, _run(g, p, t, args, form=form, max_steps=4, calls=60, pickup=1, blocks_per_sm=2, **kw))
+
+
+def test_queue_full_during_the_hand_over(oracle_lib):
+    """Slots run out while particles are handed on: parked ones resume after crp_sim_reserve."""
+    import paper_1410_5323_gb300 as crp
+
+    n = 60_000
+    p = I.make_particles(n, 18, species=MIX, energy=("power", 3e18, 10 ** 20.5, 2.0))
+    g, t, args = _grid(16, 6), I.constant_rate_tables(0.0, 1 / (3 * I.MPC)), (1e-4, I.KPC, I.MPC, 2 * I.MPC)
+    sim = crp.Simulation([crp.Field(g, 0.25 * I.MPC)], crp.Tables(t), seed=9, capacity=n + 9000)
+    sim.inject(p)
+    sim.propagate(*args)
+    assert sim.sync(60.0, raise_on_error=False) == crp.api.ERR_QUEUE_FULL
+    sim.reserve(6 * n)
+    sim.propagate(*args)
+    assert sim.sync(60.0) == 0
+    st, rc = run_oracle([g], p, t, *args, seed=9, capacity=6 * n)
+    assert rc == 0
+    assert_bit_identical(sim.state(), st.snapshot())
