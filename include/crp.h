@@ -230,10 +230,13 @@ typedef struct {
 #define CRP_ORDER_COST 2         /* lowest rigidity E/Z first: expected longest first */
 #define CRP_ORDER_GRID 3         /* by grid_id, then lowest rigidity first: concurrent particles
                                     share field realisations (cache locality over many grids) */
-#define CRP_PICKUP_DEFAULT 0     /* taken up as they come, before the rest of the work list: a secondary
-                                    inherits a low energy and can be the longest trajectory of the call */
-#define CRP_PICKUP_OFF 1         /* secondaries wait for the second launch */
-#define CRP_PICKUP_ON 2          /* idle warps take secondaries pushed earlier in the launch */
+#define CRP_PICKUP_DEFAULT 0     /* idle lanes take them up as they come, before the rest of the work list (FP64
+                                    form, lists above 12 fills of the lanes: once the list has run out), unless
+                                    more are waiting than the launch has lanes: a secondary inherits a low
+                                    energy and can be the longest trajectory of the call */
+#define CRP_PICKUP_OFF 1         /* secondaries wait for the next launch of the call */
+#define CRP_PICKUP_ON 2          /* the same once the work list has run out. A warp that holds no particle and
+                                    finds none ends; what nobody took waits for the next launch. */
 int crp_propagate(crp_sim* sim, const crp_params* params, double tolerance, double min_step_m,
                   double max_step_m, double max_distance_m, void* stream);
 

@@ -15,6 +15,7 @@ namespace crp {
 constexpr unsigned kSchedFull = 0xffffffffu;
 constexpr int kPublishWaitLimit = 1 << 22;     // iterations of 64 ns sleeps (~0.3 s)
 constexpr int kClaimRetryLimit = 64;
+constexpr int kClaimTries = 4;
 
 __device__ __forceinline__ unsigned long long ld_volatile(const unsigned long long* p) {
     return *(volatile const unsigned long long*)p;
@@ -98,21 +99,30 @@ __device__ __forceinline__ int sched_pop(const PropArgs& a, const WorkList& W, b
     return sched_slot(a, a.lists[W.L][W.back ? W.n_work - 1 - (pos - W.head0) : pos], bits, resumed);
 }
 
-// Whether idle lanes look for pushed secondaries in this turn of the one-lane kernels: now and then
-// while the list lasts, seldom once it has run out. The look is a round trip to L2, and with thousands
-// of warps asking it is the counters' line that everyone waits for (10^6 nuclei in the precision form:
-// 73 ms without pick-ups; 265, 114, 81, 66 ms looking every 1, 4, 16, 64 turns; 68 ms every 16 and, with
-// the list empty, every 128. 10^5 nuclei in the modulated scenario: 65 ms without, 44 to 47 ms with).
+// Whether idle lanes look for pushed secondaries in this turn of the one-lane kernels: every few turns,
+// with CRP_PICKUP_ON once the list has run out. The look is a round trip to L2, and with thousands of warps
+// asking it is the counters' line that everyone waits for (10^6 nuclei in the precision form: 73 ms without
+// pick-ups; 265, 114, 81, 66 ms looking every 1, 4, 16, 64 turns. 10^5 nuclei in the modulated scenario: 65 ms
+// without, 44 to 47 ms with). So that form's warps look every 32 turns, each in a turn of its own (20 000
+// nuclei over at most 200 steps 4.4 ms all at once, 2.7 so), and give up after four lost claims. Looking less
+// often once the list has run out leaves lanes idle for longer than a short flight takes (10^4 nuclei, 2 Mpc
+// between interactions, over 6 Mpc: 2.4 ms every 128 turns, 1.3 every 32).
 // The FP64 form, whose turns take ten times as long, looks every 4 (200 000 nuclei: 284 ms without,
 // 247 ms, 267 ms looking every 32).
+//
+// Where more than `room` secondaries wait, the lanes or teams of the launch, the next launch takes them: it
+// fills its lanes without asking for each (precision form, 200 000 nuclei as above 8.5 -> 4.3 ms, 10^6 20.6 ->
+// 16.9 ms; 10^5 iron nuclei 25 -> 10 ms; the limit at half the lanes: 200 000 nuclei over 100 Mpc 21.3 -> 29.5 ms,
+// since their few long secondaries then follow the list).
 template <unsigned Every>
 __device__ __forceinline__ bool sched_look(const PropArgs& a, bool dry, unsigned turn) {
-    return a.pickup && (dry ? turn % 128 == 0 : (a.pickup == 2 && turn % Every == 0));
+    return a.pickup && (dry || a.pickup == 2) && turn % Every == 0;
 }
 
 // The same from list P, into which this launch pushes secondaries only: claims positions below the
 // push count, then waits, bounded, for the entries to be published.
-__device__ __forceinline__ int sched_pick(const PropArgs& a, int P, bool idle, int lane, unsigned& bits) {
+__device__ __forceinline__ int sched_pick(const PropArgs& a, int P, unsigned long long room, bool idle, int lane,
+                                         unsigned& bits) {
     const unsigned im = __ballot_sync(kSchedFull, idle);
     if (!im) return -1;
     Counters* C = a.ctr;
@@ -121,10 +131,10 @@ __device__ __forceinline__ int sched_pick(const PropArgs& a, int P, bool idle, i
     if (lane == 0) {
         const unsigned need = (unsigned)__popc(im);
 #pragma unroll 1
-        for (int t = 0; t < kClaimRetryLimit; ++t) {
+        for (int t = 0; t < kClaimTries; ++t) {
             const unsigned long long h = ld_volatile(&C->head[P]);
             const unsigned long long c = ld_volatile(&C->count[P]);
-            if (h >= c) break;
+            if (h >= c || c - h > room) break;
             const unsigned take = (unsigned)min((unsigned long long)need, c - h);
             if (atomicCAS(&C->head[P], h, h + take) == h) {
                 base = h;
@@ -152,7 +162,8 @@ __device__ __forceinline__ int sched_pick(const PropArgs& a, int P, bool idle, i
 // before the first particle handed on. So no particle is handed on twice in one launch, which bounds the
 // length of the list (list_length). In the precision form, where all warps ask the same counters, this
 // costs 5 % (10^6 nuclei 65.4 ms claiming first, 68.8 ms reading first); the FP64 form shows no difference.
-__device__ __forceinline__ int sched_pick_secondaries(const PropArgs& a, int P, bool idle, int lane, unsigned& bits) {
+__device__ __forceinline__ int sched_pick_secondaries(const PropArgs& a, int P, unsigned long long room, bool idle, int lane,
+                                                     unsigned& bits) {
     const unsigned im = __ballot_sync(kSchedFull, idle);
     if (!im) return -1;
     Counters* C = a.ctr;
@@ -163,7 +174,7 @@ __device__ __forceinline__ int sched_pick_secondaries(const PropArgs& a, int P, 
         if (lane == 0) {
             h = ld_volatile(&C->head[P]);
             const unsigned long long c = ld_volatile(&C->count[P]);
-            if (h < c) n = (unsigned)min((unsigned long long)__popc(im), c - h);
+            if (h < c && c - h <= room) n = (unsigned)min((unsigned long long)__popc(im), c - h);
         }
         n = __shfl_sync(kSchedFull, n, 0);
         if (n == 0) return -1;

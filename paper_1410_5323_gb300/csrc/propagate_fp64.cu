@@ -88,13 +88,14 @@ __global__ void CRP_FP64_BOUNDS k_propagate_fp64(const PropArgs a) {
     // Secondaries as they come only where the list is at most 12 fills of the lanes: their long
     // trajectories are the call's tail there; in longer lists they wait for its end (10^6 nuclei, 26 fills:
     // 7173 ms as they come, 7120 at the end; 200 000, 5 fills: 247 and 284 ms).
-    const bool early = work.n_work - work.head0 <= 12ull * gridDim.x * blockDim.x;
+    const unsigned long long lanes = (unsigned long long)gridDim.x * blockDim.x;
+    const bool early = work.n_work - work.head0 <= 12 * lanes;
     bool dry = false, drain = false;
     for (unsigned turn = 0;; ++turn) {
         // ---- refill idle lanes from the work list (one atomic per warp) ----
         int popped = -1, resumed = 0;
         if (!drain && (early || dry) && sched_look<4>(a, dry, turn))
-            popped = sched_pick_secondaries(a, pushes, slot < 0, lane, bits);
+            popped = sched_pick_secondaries(a, pushes, lanes, slot < 0, lane, bits);
         if (!dry) {
             const int p = sched_pop(a, work, slot < 0 && popped < 0, lane, bits, dry, resumed);
             if (p >= 0) popped = p;

@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(256, M ? 1 : 2) k_propagate_fp64_team(const Pr
         const bool pick = a.pickup && !drain && turn % 4 == 0;
         if ((!dry && !drain) || pick) {
             int p0 = -1, resumed = 0;
-            if (pick) p0 = sched_pick_secondaries(a, pushes, first && slot < 0, lane, bits);
+            if (pick) p0 = sched_pick_secondaries(a, pushes, warps * kTeams, first && slot < 0, lane, bits);
             if (!dry && !drain) {
                 const int p = sched_pop(a, work, first && slot < 0 && p0 < 0 && lane < 3 * quota, lane, bits, dry, resumed);
                 if (p >= 0) p0 = p;
