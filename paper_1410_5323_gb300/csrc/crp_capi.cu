@@ -217,6 +217,7 @@ __global__ void k_prepare(Counters* C, int pickup) {
     C->pushed = 0;
     C->head0 = 0;
     C->left = 0;
+    C->claimed = 0;
 }
 
 // Puts -1 (nothing published) into both work lists if an earlier call left entries in them; l0 is
@@ -374,6 +375,7 @@ __global__ void k_swap(Counters* C, long long capacity, long long lo, long long 
     C->pushed = 1;
     C->head0 = C->head[1 - from];
     C->left = 0;
+    C->claimed = 0;
     C->launches += 1;
 }
 

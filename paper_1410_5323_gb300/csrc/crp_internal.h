@@ -89,6 +89,7 @@ struct Counters {
     int pushed;                      // that list was filled by a propagate launch of this call
     int tidy;                        // the work lists hold no entry of an earlier call (calls with pick-up keep them so)
     unsigned long long head0;        // first entry of that list (earlier ones were picked up when pushed)
+    unsigned long long claimed;      // pushed entries claimed by the current launch (precision form)
     unsigned long long left;         // entries of the list whose particle the current launch has stored
 };
 

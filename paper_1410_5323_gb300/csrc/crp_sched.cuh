@@ -15,7 +15,6 @@ namespace crp {
 constexpr unsigned kSchedFull = 0xffffffffu;
 constexpr int kPublishWaitLimit = 1 << 22;     // iterations of 64 ns sleeps (~0.3 s)
 constexpr int kClaimRetryLimit = 64;
-constexpr int kClaimTries = 4;
 
 __device__ __forceinline__ unsigned long long ld_volatile(const unsigned long long* p) {
     return *(volatile const unsigned long long*)p;
@@ -104,23 +103,26 @@ __device__ __forceinline__ int sched_pop(const PropArgs& a, const WorkList& W, b
 // asking it is the counters' line that everyone waits for (10^6 nuclei in the precision form: 73 ms without
 // pick-ups; 265, 114, 81, 66 ms looking every 1, 4, 16, 64 turns. 10^5 nuclei in the modulated scenario: 65 ms
 // without, 44 to 47 ms with). So that form's warps look every 32 turns, each in a turn of its own (20 000
-// nuclei over at most 200 steps 4.4 ms all at once, 2.7 so), and give up after four lost claims. Looking less
-// often once the list has run out leaves lanes idle for longer than a short flight takes (10^4 nuclei, 2 Mpc
-// between interactions, over 6 Mpc: 2.4 ms every 128 turns, 1.3 every 32).
+// nuclei over at most 200 steps 4.4 ms all at once, 2.7 so). Looking less often once the list has run out
+// leaves lanes idle for longer than a short flight takes (10^4 nuclei, 2 Mpc between interactions, over
+// 6 Mpc: 2.4 ms every 128 turns, 1.3 every 32).
 // The FP64 form, whose turns take ten times as long, looks every 4 (200 000 nuclei: 284 ms without,
 // 247 ms, 267 ms looking every 32).
 //
-// Where more than `room` secondaries wait, the lanes or teams of the launch, the next launch takes them: it
-// fills its lanes without asking for each (precision form, 200 000 nuclei as above 8.5 -> 4.3 ms, 10^6 20.6 ->
-// 16.9 ms; 10^5 iron nuclei 25 -> 10 ms; the limit at half the lanes: 200 000 nuclei over 100 Mpc 21.3 -> 29.5 ms,
-// since their few long secondaries then follow the list).
+// Where more than `room` secondaries wait, the next launch takes them: it fills its lanes without asking for
+// each. room is three times the lanes in the precision form (400 000 nuclei as above 8.4 ms without the limit,
+// 7.0 with it; 19 000 iron nuclei 9.2 and 3.5 ms; at once the lanes 300 000 nuclei over 200 Mpc 74.4 ms, with
+// their few long secondaries behind the list, 56.7 at three times) and the lanes or teams in the FP64 form.
 template <unsigned Every>
 __device__ __forceinline__ bool sched_look(const PropArgs& a, bool dry, unsigned turn) {
     return a.pickup && (dry || a.pickup == 2) && turn % Every == 0;
 }
 
-// The same from list P, into which this launch pushes secondaries only: claims positions below the
-// push count, then waits, bounded, for the entries to be published.
+// The same from list P, into which this launch pushes secondaries only: claims positions below the push
+// count, then waits, bounded, for the entries to be published. The claim is a semaphore (Counters::claimed):
+// add what is wanted, keep what the count covers, give the rest back, and take that many positions at the
+// head, which so never passes the count. No claim fails because another one came first: with a CAS on the
+// head one warp won per round trip, 30 entries a microsecond (100 000 nuclei as above 4.6 -> 2.6 ms).
 __device__ __forceinline__ int sched_pick(const PropArgs& a, int P, unsigned long long room, bool idle, int lane,
                                          unsigned& bits) {
     const unsigned im = __ballot_sync(kSchedFull, idle);
@@ -129,18 +131,14 @@ __device__ __forceinline__ int sched_pick(const PropArgs& a, int P, unsigned lon
     unsigned long long base = 0;
     unsigned got = 0;
     if (lane == 0) {
-        const unsigned need = (unsigned)__popc(im);
-#pragma unroll 1
-        for (int t = 0; t < kClaimTries; ++t) {
-            const unsigned long long h = ld_volatile(&C->head[P]);
-            const unsigned long long c = ld_volatile(&C->count[P]);
-            if (h >= c || c - h > room) break;
-            const unsigned take = (unsigned)min((unsigned long long)need, c - h);
-            if (atomicCAS(&C->head[P], h, h + take) == h) {
-                base = h;
-                got = take;
-                break;
-            }
+        const unsigned long long c = ld_volatile(&C->count[P]);
+        unsigned long long taken = ld_volatile(&C->claimed);
+        if (taken < c && c - taken <= room) {
+            const unsigned long long want = min((unsigned long long)__popc(im), c - taken);
+            taken = atomicAdd(&C->claimed, want);
+            got = taken < c ? (unsigned)min(want, c - taken) : 0u;
+            if (got < want) atomicAdd(&C->claimed, got - want);
+            if (got) base = atomicAdd(&C->head[P], (unsigned long long)got);
         }
     }
     base = __shfl_sync(kSchedFull, base, 0);
