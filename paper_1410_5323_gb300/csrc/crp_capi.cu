@@ -1497,23 +1497,26 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
         int occ = prm->blocks_per_sm;
         if (occ <= 0 && (propagate_team_occupancy(s->mod, p2, block, &occ) != 0 || occ < 1)) occ = 1;
         P.team_grid = sms * std::min(occ, kThreadsPerSm / block);
-        const long long layer = (long long)sms * (block / 32) * kTeamsPerWarp;   // particles of STEP_LAYER
+        const long long layer = (long long)sms * (block / 32) * kTeamsPerWarp;   // teams of STEP_LAYER
+        // Up to three particles a team, one block per SM is still the better one (tables, over 50 Mpc: 10 000
+        // nuclei 54.6 ms in several blocks per SM, 24.4 in one; 20 000 take 43 ms in several).
+        const long long few = 3 * layer;
         // Handed on by STEP_FULL once half of the lanes hold a particle: full lanes are worth more than teams
         // (10^6 nuclei over 500 Mpc: 7473 ms handing on as soon as the list has run out, 7173 at 6/8 or
         // less; 10^6 in a modulated field 5598 at 6/8, 5506 at 4/8, 5513 never; 60 000 over 100 Mpc: 285
         // without teams, 141 at once, 138 at 6/8, 140 at 4/8, 147 at 2/8), by STEP_TEAM once one block per SM
         // holds them.
         const long long to_team = s->taken ? lanes / 2 : -1, to_layer = s->taken ? layer : -1;
-        if (s->tables && cap > layer) {
-            step(STEP_LAYER, -1, layer);
-            step(STEP_TEAM, layer, cap > lanes ? lanes : kAny, to_layer);
+        if (s->tables && cap > few) {
+            step(STEP_LAYER, -1, few);
+            step(STEP_TEAM, few, cap > lanes ? lanes : kAny, to_layer);
         }
         if (cap > lanes) {
             step(STEP_FULL, lanes, kAny, to_team);
             if (s->tables) step(STEP_FULL, lanes, kAny, to_team);
         }
-        if (cap > layer && (cap > lanes || !s->tables)) step(STEP_TEAM, layer, kAny, to_layer);
-        if (cap <= layer || s->tables) step(STEP_LAYER, -1, kAny);
+        if (cap > few && (cap > lanes || !s->tables)) step(STEP_TEAM, few, kAny, to_layer);
+        if (cap <= few || s->tables) step(STEP_LAYER, -1, kAny);
         step(STEP_LAYER, -1, kAny);
     } else if (mixed && prm->blocks_per_sm <= 0) {
         // lists that fit one block per SM go to launches of that shape, which deal the particles out evenly

@@ -2,7 +2,7 @@
 // its idle lanes with one claim on a global counter (ballot + popc), first from the fixed
 // work list of the launch, then from the list of secondaries pushed during this launch.
 // A pushed entry is published with a release store after the particle's state is written;
-// a reader claims entries below the push count with a CAS and waits, bounded, for each to
+// a reader claims entries below the push count and waits, bounded, for each to
 // appear with an acquire load. A wait that runs out sets a status bit instead of hanging;
 // nothing here traps.
 #pragma once

@@ -244,3 +244,12 @@ def test_queue_full_during_the_hand_over(oracle_lib):
     st, rc = run_oracle([g], p, t, *args, seed=9, capacity=6 * n)
     assert rc == 0
     assert_bit_identical(sim.state(), st.snapshot())
+
+
+@pytest.mark.parametrize("tables", [False, True])
+@pytest.mark.parametrize("n", [18_240, 18_241, 38_912, 38_913])
+def test_batches_around_three_layers_and_the_lanes(oracle_lib, n, tables):
+    """One block per SM up to three particles a team, several up to the one-lane kernel's lanes."""
+    p = I.make_particles(n, 19, species=MIX, energy=("power", 3e18, 10 ** 20.5, 2.0))
+    t = I.constant_rate_tables(1 / (200 * I.MPC), 1 / (3 * I.MPC)) if tables else None
+    _same([_grid(16, 5)], p, t, 1e-4, I.KPC, I.MPC, I.MPC, seed=n, capacity=4 * n if tables else n)
