@@ -232,8 +232,8 @@ typedef struct {
                                     share field realisations (cache locality over many grids) */
 #define CRP_PICKUP_DEFAULT 0     /* idle lanes take them up as they come, before the rest of the work list (FP64
                                     form, lists above 12 fills of the lanes: once the list has run out), unless
-                                    so many are waiting that the next launch of the call will be full: a
-                                    secondary inherits a low energy and can be the longest trajectory */
+                                    so many are waiting that they are the next launch's: a secondary inherits
+                                    a low energy and can be the longest trajectory */
 #define CRP_PICKUP_OFF 1         /* secondaries wait for the next launch of the call */
 #define CRP_PICKUP_ON 2          /* the same once the work list has run out. A warp that holds no particle and
                                     finds none ends; what nobody took waits for the next launch. */

@@ -214,7 +214,8 @@ __global__ void k_prepare(Counters* C, int pickup) {
     C->head[1] = 0;
     C->reserve = C->n_used;
     C->cur = 0;
-    C->pushed = 0;
+    C->handed = 0;
+    C->handed0 = 0;
     C->head0 = 0;
     C->left = 0;
     C->claimed = 0;
@@ -372,7 +373,8 @@ __global__ void k_swap(Counters* C, long long capacity, long long lo, long long 
     C->head[from] = 0;      // the other list keeps its head: the next launch continues it
     C->count[from] = 0;
     C->cur = 1 - from;
-    C->pushed = 1;
+    C->handed0 = C->handed;
+    C->handed = 0;
     C->head0 = C->head[1 - from];
     C->left = 0;
     C->claimed = 0;
@@ -1560,7 +1562,6 @@ int make_plan(crp_sim* s, const crp_params* prm, double tol, double hmin, double
     a.spread = 0;
     a.drain = 0;
     a.taken = team ? s->taken : nullptr;
-    a.back = team ? 1 : 0;
     a.lists[0] = s->lists[0];
     a.lists[1] = s->lists[1];
     a.done_list = s->done_list;

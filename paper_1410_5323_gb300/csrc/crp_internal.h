@@ -86,9 +86,11 @@ struct Counters {
     unsigned long long prev_accepted;
     unsigned int status_bits;
     int cur;                         // work list (0 or 1) that the next propagate launch takes
-    int pushed;                      // that list was filled by a propagate launch of this call
+    int pad_;
     int tidy;                        // the work lists hold no entry of an earlier call (calls with pick-up keep them so)
     unsigned long long head0;        // first entry of that list (earlier ones were picked up when pushed)
+    unsigned long long handed;       // particles handed on by the current launch
+    unsigned long long handed0;      // entries of the list that are particles handed on
     unsigned long long claimed;      // pushed entries claimed by the current launch (precision form)
     unsigned long long left;         // entries of the list whose particle the current launch has stored
 };
@@ -110,7 +112,7 @@ struct PropArgs {
     int32_t pad2_;
     int32_t drain;                   // once the list has run out and at most drain_at particles are left, hand
                                      // active particles on to the next launch
-    int32_t back;                    // lists that a launch of this call filled are taken from their end
+    int32_t pad3_;
     long long drain_at;
     long long min_work, max_work;    // a launch takes lists of more than min_work and at most max_work entries
                                      // and leaves others to the next one

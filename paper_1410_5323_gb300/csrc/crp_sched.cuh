@@ -44,8 +44,14 @@ __device__ __forceinline__ void sched_push(const PropArgs& a, int L, int32_t q) 
 // of the call handed on; -1: not yet published (the bookkeeping after each launch puts it back).
 constexpr int32_t kResumed = -2;
 
+__device__ __forceinline__ void sched_hand_on(const PropArgs& a, int L, int32_t slot) {
+    atomicAdd(&a.ctr->handed, 1ull);
+    sched_push(a, L, kResumed - slot);
+}
+
+template <bool HandedOn>
 __device__ __forceinline__ int sched_slot(const PropArgs& a, int32_t v, unsigned& bits, int& resumed) {
-    if (v <= kResumed && a.taken) {
+    if (HandedOn && v <= kResumed && a.taken) {
         v = kResumed - v;
         resumed = 1;
     }
@@ -54,12 +60,13 @@ __device__ __forceinline__ int sched_slot(const PropArgs& a, int32_t v, unsigned
 }
 
 // What a launch works through: list L from position head0 (entries before it were taken by the
-// previous launch) to n_work. back: from the end (a list that a launch filled ends with the
-// particles handed on, the long ones).
+// previous launch) to n_work. A list that a launch filled ends with the particles it handed on, which are
+// in mid-flight: as many entries as those, from the end, come first, then the secondaries in the order in
+// which they were released, lowest rigidities first. (All from the end, with the longest secondaries
+// last, 10^6 nuclei over 500 Mpc took 7.50 s instead of 7.04.)
 struct WorkList {
     int L;
-    bool back;
-    unsigned long long n_work, head0;
+    unsigned long long from_end, n_work, head0;
     __device__ __forceinline__ bool fits(const PropArgs& a) const {
         const long long n = (long long)(n_work - head0);
         return n > a.min_work && n <= a.max_work;
@@ -68,11 +75,13 @@ struct WorkList {
 __device__ __forceinline__ WorkList work_list(const PropArgs& a) {
     const Counters* C = a.ctr;
     const int L = *(volatile const int*)&C->cur;
-    return {L, a.back && *(volatile const int*)&C->pushed, ld_volatile(&C->count[L]), ld_volatile(&C->head0)};
+    return {L, ld_volatile(&C->handed0), ld_volatile(&C->count[L]), ld_volatile(&C->head0)};
 }
 
 // Returns the slot this lane should load next from the work list, or -1. Lanes with idle == false
-// get -1. dry (the same in all lanes) turns true once the list has run out for good.
+// get -1. dry (the same in all lanes) turns true once the list has run out for good. HandedOn: the list may
+// hold particles handed on (FP64 form; the precision kernels have no registers to spare for them).
+template <bool HandedOn>
 __device__ __forceinline__ int sched_pop(const PropArgs& a, const WorkList& W, bool idle, int lane, unsigned& bits,
                                         bool& dry, int& resumed) {
     const unsigned im = __ballot_sync(kSchedFull, idle);
@@ -94,8 +103,12 @@ __device__ __forceinline__ int sched_pop(const PropArgs& a, const WorkList& W, b
     if (!idle) return -1;
     const unsigned rank = (unsigned)__popc(im & ((1u << lane) - 1u));
     if (rank >= got) return -1;
-    const unsigned long long pos = base + rank;
-    return sched_slot(a, a.lists[W.L][W.back ? W.n_work - 1 - (pos - W.head0) : pos], bits, resumed);
+    unsigned long long pos = base + rank;
+    if constexpr (HandedOn) {
+        const unsigned long long k = pos - W.head0;
+        pos = k < W.from_end ? W.n_work - 1 - k : pos - W.from_end;
+    }
+    return sched_slot<HandedOn>(a, a.lists[W.L][pos], bits, resumed);
 }
 
 // Whether idle lanes look for pushed secondaries in this turn of the one-lane kernels: every few turns,
@@ -103,27 +116,29 @@ __device__ __forceinline__ int sched_pop(const PropArgs& a, const WorkList& W, b
 // asking it is the counters' line that everyone waits for (10^6 nuclei in the precision form: 73 ms without
 // pick-ups; 265, 114, 81, 66 ms looking every 1, 4, 16, 64 turns. 10^5 nuclei in the modulated scenario: 65 ms
 // without, 44 to 47 ms with). So that form's warps look every 32 turns, each in a turn of its own (20 000
-// nuclei over at most 200 steps 4.4 ms all at once, 2.7 so). Looking less often once the list has run out
-// leaves lanes idle for longer than a short flight takes (10^4 nuclei, 2 Mpc between interactions, over
-// 6 Mpc: 2.4 ms every 128 turns, 1.3 every 32).
+// nuclei over at most 200 steps 4.4 ms all at once, 2.7 so), and every 4 once the list has run out, where
+// lanes without a particle have nothing else to do (200 000 nuclei, 2 Mpc between interactions, over 6 Mpc:
+// 9.2 ms every 128 turns, 4.5 every 32, 3.8 every 4).
 // The FP64 form, whose turns take ten times as long, looks every 4 (200 000 nuclei: 284 ms without,
 // 247 ms, 267 ms looking every 32).
 //
-// Where more than `room` secondaries wait, the next launch takes them: it fills its lanes without asking for
-// each. room is three times the lanes in the precision form (400 000 nuclei as above 8.4 ms without the limit,
-// 7.0 with it; 19 000 iron nuclei 9.2 and 3.5 ms; at once the lanes 300 000 nuclei over 200 Mpc 74.4 ms, with
-// their few long secondaries behind the list, 56.7 at three times) and the lanes or teams in the FP64 form.
-template <unsigned Every>
+// Where too many secondaries wait, the next launch takes them: it fills its lanes without asking for each.
+// In the precision form that is three times the lanes for lists that don't fill the lanes (30 000 iron
+// nuclei 3.4 ms without a limit, 2.4 with it; 19 000 in one block per SM 5.3 and 1.5), and no limit for longer
+// lists, whose tail the secondaries fill (10^6 nuclei over 500 Mpc 396 ms; 420 with the limit, the secondaries'
+// own tail behind the nuclei's); in the FP64 form, whose tail other launches take, the lanes or teams.
+template <unsigned Every, unsigned Dry>
 __device__ __forceinline__ bool sched_look(const PropArgs& a, bool dry, unsigned turn) {
-    return a.pickup && (dry || a.pickup == 2) && turn % Every == 0;
+    return a.pickup && (dry ? turn % Dry == 0 : (a.pickup == 2 && turn % Every == 0));
 }
 
 // The same from list P, into which this launch pushes secondaries only: claims positions below the push
 // count, then waits, bounded, for the entries to be published. The claim is a semaphore (Counters::claimed):
 // add what is wanted, keep what the count covers, give the rest back, and take that many positions at the
 // head, which so never passes the count. No claim fails because another one came first: with a CAS on the
-// head one warp won per round trip, 30 entries a microsecond (100 000 nuclei as above 4.6 -> 2.6 ms).
-__device__ __forceinline__ int sched_pick(const PropArgs& a, int P, unsigned long long room, bool idle, int lane,
+// head one warp won per round trip, 30 entries a microsecond (100 000 nuclei as above, looking every 32 turns,
+// 4.6 -> 2.6 ms).
+__device__ __forceinline__ int sched_pick(const PropArgs& a, int P, unsigned long long n_work, bool idle, int lane,
                                          unsigned& bits) {
     const unsigned im = __ballot_sync(kSchedFull, idle);
     if (!im) return -1;
@@ -131,9 +146,10 @@ __device__ __forceinline__ int sched_pick(const PropArgs& a, int P, unsigned lon
     unsigned long long base = 0;
     unsigned got = 0;
     if (lane == 0) {
-        const unsigned long long c = ld_volatile(&C->count[P]);
+        const unsigned long long c = ld_volatile(&C->count[P]), lanes = (unsigned long long)gridDim.x * blockDim.x;
+        const bool fills = n_work - ld_volatile(&C->head0) > lanes;
         unsigned long long taken = ld_volatile(&C->claimed);
-        if (taken < c && c - taken <= room) {
+        if (taken < c && (fills || c - taken <= 3 * lanes)) {
             const unsigned long long want = min((unsigned long long)__popc(im), c - taken);
             taken = atomicAdd(&C->claimed, want);
             got = taken < c ? (unsigned)min(want, c - taken) : 0u;
@@ -152,7 +168,7 @@ __device__ __forceinline__ int sched_pick(const PropArgs& a, int P, unsigned lon
         return -1;
     }
     int resumed = 0;
-    return sched_slot(a, v, bits, resumed);
+    return sched_slot<false>(a, v, bits, resumed);
 }
 
 // The same where the list also receives particles handed on to the next launch (FP64 form). The warp

@@ -94,10 +94,10 @@ __global__ void CRP_FP64_BOUNDS k_propagate_fp64(const PropArgs a) {
     for (unsigned turn = 0;; ++turn) {
         // ---- refill idle lanes from the work list (one atomic per warp) ----
         int popped = -1, resumed = 0;
-        if (!drain && (early || dry) && sched_look<4>(a, dry, turn))
+        if (!drain && (early || dry) && sched_look<4, 4>(a, dry, turn))
             popped = sched_pick_secondaries(a, pushes, lanes, slot < 0, lane, bits);
         if (!dry) {
-            const int p = sched_pop(a, work, slot < 0 && popped < 0, lane, bits, dry, resumed);
+            const int p = sched_pop<true>(a, work, slot < 0 && popped < 0, lane, bits, dry, resumed);
             if (p >= 0) popped = p;
             if (a.drain && turn % 8 == 7) {   // a full warp asks for nothing: look whether the list has run out
                 unsigned long long head = lane == 0 ? ld_volatile(&C->head[work.L]) : 0ull;
@@ -114,7 +114,7 @@ __global__ void CRP_FP64_BOUNDS k_propagate_fp64(const PropArgs a) {
             const int32_t q = slot;
             a.taken[q] = (int32_t)taken;
             store(CRP_STATUS_ACTIVE_);
-            sched_push(a, pushes, kResumed - q);
+            sched_hand_on(a, pushes, q);
         }
         if (popped >= 0) {
             slot = popped;

@@ -424,9 +424,9 @@ __device__ __forceinline__ void propagate_mixed_body(const PropArgs& a, float* s
     bool dry = false;
     for (unsigned turn = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;; ++turn) {   // each warp looks in its own turns
         int popped = -1, resumed = 0;
-        if (PICK && sched_look<32>(a, dry, turn)) popped = sched_pick(a, pushes, 3 * 32 * warps, slot < 0, lane, bits);
+        if (PICK && sched_look<32, 4>(a, dry, turn)) popped = sched_pick(a, pushes, work.n_work, slot < 0, lane, bits);
         if (!dry) {
-            const int p = sched_pop(a, work, slot < 0 && popped < 0 && lane < quota, lane, bits, dry, resumed);
+            const int p = sched_pop<false>(a, work, slot < 0 && popped < 0 && lane < quota, lane, bits, dry, resumed);
             if (p >= 0) popped = p;
         }
         if (popped >= 0) {

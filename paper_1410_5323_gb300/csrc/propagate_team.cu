@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(256, M ? 1 : 2) k_propagate_fp64_team(const Pr
             int p0 = -1, resumed = 0;
             if (pick) p0 = sched_pick_secondaries(a, pushes, warps * kTeams, first && slot < 0, lane, bits);
             if (!dry && !drain) {
-                const int p = sched_pop(a, work, first && slot < 0 && p0 < 0 && lane < 3 * quota, lane, bits, dry, resumed);
+                const int p = sched_pop<true>(a, work, first && slot < 0 && p0 < 0 && lane < 3 * quota, lane, bits, dry, resumed);
                 if (p >= 0) p0 = p;
             }
             const int popped = T.get(p0, 0);
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(256, M ? 1 : 2) k_propagate_fp64_team(const Pr
                 const int32_t q = slot;
                 if (T.c == 0) a.taken[q] = (int32_t)taken;
                 store(CRP_STATUS_ACTIVE_);
-                if (T.c == 0) sched_push(a, pushes, kResumed - q);
+                if (T.c == 0) sched_hand_on(a, pushes, q);
             }
             __syncwarp();
         }
