@@ -71,11 +71,13 @@ MOD_FLOP_PER_ACCEPTED = 42
 MIXED_MOD_FP64_OPS_PER_ACCEPTED = 33
 MIXED_MOD_FP32_FLOP_PER_ATTEMPT = 228
 # DRAM bytes (read + write) per attempted step of the propagate kernels, measured by ncu at
-# reduced batch (both launches of one call; the summaries under profiles/ name the command);
-# traffic of a call = this x its attempts. Keyed by (workload, form).
+# reduced batch (all launches of one call; the summaries under profiles/ name the command);
+# traffic of a call = this x its attempts. Keyed by (workload, form). The first two were measured
+# with the nuclei and their secondaries in a launch each; with the present launches 144.5 and 101.1.
 DRAM_BYTES_PER_ATTEMPT = {("fp64_256cube_1M_nuclei", "fp64"): 139.1,
                           ("fp64_256cube_1M_nuclei", "mixed"): 99.3,      # cell-major grid copy
-                          ("modulated_440cube_300kpc_x_256cube_50kpc_1M_nuclei", "fp64"): 372.8}
+                          ("modulated_440cube_300kpc_x_256cube_50kpc_1M_nuclei", "fp64"): 406.6,
+                          ("modulated_440cube_300kpc_x_256cube_50kpc_1M_nuclei", "mixed"): 465.5}
 
 
 def parse():
@@ -435,7 +437,7 @@ def roofline_for(form, attempted, accepted, tables, prop_s, calls=1, workload=""
     terms = roofline_terms(form, attempted, accepted, tables, prop_s, modulated, grid_dtype,
                            grid_bytes, peaks)
     kern = ("k_propagate_fp64, then k_propagate_fp64_team for what is left" if form == "fp64" else
-            "k_propagate_mixed, two launches") + " (and the bookkeeping kernels of a call)"
+            "k_propagate_mixed, a launch for the list and more for what it leaves") + " (and the bookkeeping kernels of a call)"
     return roofline_from_terms(terms, traffic_for(workload, form, attempted, calls), kern, note)
 
 
@@ -1000,7 +1002,7 @@ def run_adjoint(args):
     roof = roofline_from_terms(terms, None,
                                "k_adj_record_team + k_adj_records + k_adj_reverse_team (+ init, p0-bar)",
                                note=f"{n} independent chains: three lanes per chain (one per axis) in the "
-                                    "serial record and reverse sweeps, one thread per (chain, segment) "
+                                    "serial record and reverse sweeps, one thread per (chain, step) "
                                     "in the stage records")
 
     # ---- end to end: inputs from pinned host memory, gradients back ----
