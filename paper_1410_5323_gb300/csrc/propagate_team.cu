@@ -12,9 +12,10 @@
 // last launches of 200 000 nuclei 363 -> 244 ms.
 //
 // A call runs the one-lane kernel on work lists of more entries than it has lanes (38 912 here); when
-// its list has run out and half of its lanes are empty it hands its particles on. Then this
-// kernel with several blocks per SM, which hands on once one block per SM can hold what is left, and
-// with one block per SM to the end: warps that share a sub-partition share its FP64 unit.
+// its list has run out and half of its lanes are empty it hands its particles on. Lists of more than three
+// particles for each team of one block per SM (18 240) go to this kernel with several blocks per SM, which
+// hands on once one block per SM can hold what is left, and the rest runs with one block per SM to the end:
+// warps that share a sub-partition share its FP64 unit.
 #include <cuda_runtime.h>
 
 #include "crp_internal.h"
